@@ -381,10 +381,11 @@ int read_common(vista_stack *h, void *sum_wv, void *sum_w, void *sum_wvv, uint32
     if (e != cudaSuccess) return cuda_fail(h, e, "error word read");
     if (err != 0) return device_fail(h, err);
     const int fp64 = h->desc.precision == VISTA_PREC_FP64;
+    const int all = cube_counts_exact(h) ? 0 : 1;
     const int64_t n = h->nentries;
     const size_t fe = out_f64 ? 8 : 4;
     if (dst_dev) {
-        e = launch_unpack(h->cube, h->cube_master, h->count, fp64, n, sum_wv, sum_w, sum_wvv, count, out_f64,
+        e = launch_unpack(h->cube, h->cube_master, h->count, fp64, all, n, sum_wv, sum_w, sum_wvv, count, out_f64,
                           h->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "cube unpack");
@@ -400,7 +401,7 @@ int read_common(vista_stack *h, void *sum_wv, void *sum_w, void *sum_wvv, uint32
     char *d_w = sum_w ? p + b_wv : nullptr;
     char *d_vv = sum_wvv ? p + b_wv + b_w : nullptr;
     uint32_t *d_c = count ? (uint32_t *)(p + b_wv + b_w + b_vv) : nullptr;
-    e = launch_unpack(h->cube, h->cube_master, h->count, fp64, n, d_wv, d_w, d_vv, d_c, out_f64, h->stream);
+    e = launch_unpack(h->cube, h->cube_master, h->count, fp64, all, n, d_wv, d_w, d_vv, d_c, out_f64, h->stream);
     // the four arrays go back on the copy streams, in parallel
     if (e == cudaSuccess) e = xfer_fork(h);
     if (e == cudaSuccess && sum_wv) e = cudaMemcpyAsync(sum_wv, d_wv, b_wv, cudaMemcpyDeviceToHost, h->xfer[0]);
@@ -439,6 +440,7 @@ extern "C" int vista_read_cube_async(vista_stack *h, float *sum_wv, float *sum_w
     if (e == cudaSuccess && !h->rb_done) e = cudaEventCreateWithFlags(&h->rb_done, cudaEventDisableTiming);
     if (e != cudaSuccess) return cuda_fail(h, e, "readback stream");
     const int fp64 = h->desc.precision == VISTA_PREC_FP64;
+    const int all = cube_counts_exact(h) ? 0 : 1;
     const int64_t n = h->nentries;
     const size_t b_wv = sum_wv ? (size_t)n * 8 : 0, b_w = sum_w ? (size_t)n * 4 : 0,
                  b_vv = sum_wvv ? (size_t)n * 4 : 0, b_c = count ? (size_t)n * 4 : 0;
@@ -456,7 +458,7 @@ extern "C" int vista_read_cube_async(vista_stack *h, float *sum_wv, float *sum_w
     // follows the runs queued so far on the handle's stream
     if (h->rb_pending) e = cudaStreamWaitEvent(h->stream, h->rb_done, 0);
     if (e == cudaSuccess)
-        e = launch_unpack(h->cube, h->cube_master, h->count, fp64, n, d_wv, d_w, d_vv, d_c, 0, h->stream);
+        e = launch_unpack(h->cube, h->cube_master, h->count, fp64, all, n, d_wv, d_w, d_vv, d_c, 0, h->stream);
     if (e == cudaSuccess) e = cudaEventRecord(h->rb_ready, h->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->rb_stream, h->rb_ready, 0);
     if (e == cudaSuccess && sum_wv) e = cudaMemcpyAsync(sum_wv, d_wv, b_wv, cudaMemcpyDeviceToHost, h->rb_stream);
@@ -579,15 +581,21 @@ extern "C" int vista_get_h2d_bytes(vista_stack *h, int64_t *out)
 extern "C" int vista_zero_cube(vista_stack *h)
 {
     CHECK_HANDLE(h);
-    const size_t esz = h->desc.precision == VISTA_PREC_FP64 ? 32 : 16;
-    cudaError_t e = cudaMemsetAsync(h->cube, 0, (size_t)h->nentries * esz, h->stream);
-    if (e == cudaSuccess && h->cube_master)
-        e = cudaMemsetAsync(h->cube_master, 0, (size_t)h->nentries * 32, h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->count, 0, (size_t)h->nentries * 4, h->stream);
+    const bool fp64 = h->desc.precision == VISTA_PREC_FP64;
+    cudaError_t e;
+    if (cube_counts_exact(h)) {
+        e = launch_zero_touched(h->cube, h->cube_master, h->count, fp64, h->nentries, h->stream);
+    } else {
+        e = cudaMemsetAsync(h->cube, 0, (size_t)h->nentries * (fp64 ? 32 : 16), h->stream);
+        if (e == cudaSuccess && h->cube_master)
+            e = cudaMemsetAsync(h->cube_master, 0, (size_t)h->nentries * 32, h->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(h->count, 0, (size_t)h->nentries * 4, h->stream);
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(h->stats, 0, sizeof(DevStats), h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "cube zeroing");
     h->host_nvis = 0;
     h->nvis_since_fold = 0;
+    h->count_bound = 0;
     return VISTA_OK;
 }
 

@@ -1,0 +1,70 @@
+// Device helpers for kernels that walk the cube's entries (readback, zeroing,
+// continuum subtraction): float-pair arithmetic that stays off the FP64 pipe
+// (about two lanes a clock and SM on GB300: widening, adding and narrowing the
+// four sums of every entry of a 6.7e7-entry cube took 1.3 ms there, three
+// times its memory time), and 32-byte accesses.
+#pragma once
+#include <cstdint>
+
+#include <cuda_runtime.h>
+
+namespace vista {
+
+// Four doubles of one cube entry (32-byte aligned) in one access.
+struct Double4 {
+    double x, y, z, w;
+};
+__device__ __forceinline__ Double4 load_double4(const double *p)
+{
+    Double4 d;
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(d.x), "=d"(d.y), "=d"(d.z), "=d"(d.w) : "l"(p));
+    return d;
+}
+__device__ __forceinline__ void store_zero32(void *p)
+{
+    asm volatile("st.global.v4.b64 [%0], {%1, %1, %1, %1};" ::"l"(p), "l"(0ll) : "memory");
+}
+
+// A double as hi + lo, two floats: hi is the double truncated to 24
+// significant bits, lo the remaining 29 bits rounded to a float (so hi + lo
+// is the double to about 2^-47 relative, less where lo falls below the
+// normal floats).  Integer and FP32 operations only.  Magnitudes outside
+// [2^-126, 2^128) give (0, 0): zero, and values far below any sum of
+// weights or visibilities (no sum reaches the upper end).
+__device__ __forceinline__ float2 split_double(double d)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+    const int e = (int)((b >> 52) & 0x7ff);
+    if (e < 897 || e > 1150) return make_float2(0.f, 0.f);
+    const unsigned sign = (unsigned)(b >> 63) << 31;
+    const unsigned hi_bits = sign | ((unsigned)(e - 896) << 23) | (unsigned)((b >> 29) & 0x7fffffu);
+    // the low 29 mantissa bits times 2^-52 (exact), times 2^(e - 1023)
+    const float lo = (__uint2float_rn((unsigned)(b & 0x1fffffffu)) * 0x1p-52f) * __int_as_float((e - 896) << 23);
+    return make_float2(__uint_as_float(hi_bits), sign ? -lo : lo);
+}
+
+__device__ __forceinline__ float2 add_ff(float2 a, float b)   // (a.x + a.y) + b as a pair
+{
+    const float t = a.x + b, z = t - a.x;
+    const float err = (a.x - (t - z)) + (b - z);
+    const float lo = a.y + err, hi = t + lo;
+    return make_float2(hi, lo - (hi - t));
+}
+
+static __device__ __noinline__ float sum_f32_slow(float c, double m) { return (float)((double)c + m); }
+
+// fl32(c + m) of an entry's FP32 partial and FP64 master sum (within 2^-40 of
+// a unit in the last place of the rounded FP64 sum).  Masters outside the
+// normal floats' range (infinities and NaNs among them) take the FP64 form.
+__device__ __forceinline__ float sum_f32(float c, double m)
+{
+    const int e = (__double2hiint(m) >> 20) & 0x7ff;
+    if (e == 0) return c;   // zero, or below 2^-1022
+    if (__builtin_expect(e < 897 || e > 1150, 0)) return sum_f32_slow(c, m);
+    const float2 s = split_double(m);
+    const float t = s.x + c;
+    if (!(fabsf(t) < __int_as_float(0x7f800000))) return t;   // c infinite or NaN, or an overflow
+    return add_ff(s, c).x;
+}
+
+}  // namespace vista

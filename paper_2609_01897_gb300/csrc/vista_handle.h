@@ -95,6 +95,8 @@ struct vista_stack {
     vista::DevStats *stats = nullptr;
     uint64_t host_nvis = 0;   // visibilities read, counted from the channel tables at each run
     uint64_t nvis_since_fold = 0;   // mixed: visibilities stacked since the FP32 partials were last folded
+    // the largest count any cube entry can have reached since the cube was zeroed (see entry_bound())
+    uint64_t count_bound = 0;
     int32_t *err = nullptr;
     vista::DevBuf b_srcs, b_chf, b_chd, b_recs, b_cells, b_off, b_stage, b_unpack, b_sort, b_rot, b_guvw, b_regrid,
         b_contsub, b_sparse;
@@ -121,7 +123,7 @@ struct vista_stack {
     bool graphs = true;
     bool plan_valid = false;             // device tables hold the plan of `plan_sig`
     std::vector<uint8_t> plan_sig;
-    uint64_t plan_nvis = 0;
+    uint64_t plan_nvis = 0, plan_bound = 0;
     cudaStream_t cap_stream = nullptr;   // capture stream (handle-owned)
     // host<->device copies spread over several streams (copy engines run in
     // parallel), forked from and joined back into `stream`
@@ -149,6 +151,10 @@ int device_fail(vista_stack *h, int32_t code);
 int span_begin(vista_stack *h, int kind);
 void span_end(vista_stack *h, int id);
 size_t vis_elem_bytes(int vt);
+// Whether an entry with count 0 has surely had no contribution: no 32-bit
+// count can have wrapped around to 0.  Readback, zeroing and continuum
+// subtraction then leave the sums of such entries alone.
+inline bool cube_counts_exact(const vista_stack *h) { return h->count_bound <= 0xffffffffull; }
 uint64_t freq_digest(const double *f, size_t n);   // change detection of a frequency axis
 void drop_graph(vista_stack *h);
 constexpr int NXFER = 4;

@@ -233,9 +233,12 @@ cudaError_t launch_fp64(const RunArgs &a, cudaStream_t st);
 cudaError_t launch_rotate(const RunArgs &a, cudaStream_t st);
 // Mixed cube: move every FP32 partial into the FP64 master and clear it.
 cudaError_t launch_fold(void *cube, double *master, int64_t n, cudaStream_t st);
-cudaError_t launch_unpack(const void *cube, const double *master, const uint32_t *count, int fp64, int64_t n,
+// Cube -> caller arrays; all = 1 reads every entry's sums, also where its count is 0.
+cudaError_t launch_unpack(const void *cube, const double *master, const uint32_t *count, int fp64, int all, int64_t n,
                           void *sum_wv, void *sum_w, void *sum_wvv, uint32_t *cnt_out,
                           int out_f64, cudaStream_t st);
+// Zero the entries whose count is not 0 (all others must be zero).
+cudaError_t launch_zero_touched(void *cube, double *master, uint32_t *count, int fp64, int64_t n, cudaStream_t st);
 // Sparse readback (the entries with count > 0, in entry order): per tile of
 // 4096 entries the touched count (tile_cnt [ntile]), their exclusive scan
 // (tile_off [ntile]) and the total (one int64 on the device); then each

@@ -29,6 +29,7 @@ struct Plan {
     int32_t key_ch = 0;       // in-cube channel with the largest |frequency|
     bool linear = true;
     double step = 0.0;
+    int32_t bin_ch = 0;       // the largest number of channels that touch one rest bin
     std::vector<ChanF> chf;
     std::vector<ChanD> chd;
 };
@@ -88,7 +89,25 @@ int plan_source(vista_stack *h, const SrcHost &s, double gu, double gv, Plan &pl
             pl.key_ch = k;
         }
     }
+    // channels per bin, from a difference array over the bins
+    std::vector<int32_t> open((size_t)h->desc.nrest + 1, 0);
+    for (int32_t k = lo; k < hi; ++k)
+        if (nb[(size_t)k] > 0) {
+            ++open[(size_t)j0[(size_t)k]];
+            --open[(size_t)j0[(size_t)k] + nb[(size_t)k]];
+        }
+    for (int32_t j = 0, n_open = 0; j < h->desc.nrest; ++j) pl.bin_ch = std::max(pl.bin_ch, n_open += open[(size_t)j]);
     return VISTA_OK;
+}
+
+// A bound on what one run adds to any entry's count: per window, its rows
+// times the channels that share a rest bin times the pols that share a plane.
+uint64_t entry_bound(const SrcHost &s, const Plan &pl)
+{
+    int share[VISTA_MAX_POL] = {}, most = 0;
+    for (int p = 0; p < s.d.npol; ++p)
+        if (s.pol_map[(size_t)p] >= 0) most = std::max(most, ++share[s.pol_map[(size_t)p]]);
+    return (uint64_t)s.d.nrow * (uint64_t)pl.bin_ch * (uint64_t)most;
 }
 
 // A run's table uploads go through one half of the handle's pinned staging
@@ -377,6 +396,7 @@ extern "C" int vista_run(vista_stack *h)
                 return cuda_fail(h, e, "graph capture of the device pass");
             }
         }
+        h->count_bound += h->plan_bound;
         if ((e = cudaGraphLaunch(h->gexec, h->stream)) != cudaSuccess) return cuda_fail(h, e, "graph launch");
         if ((e = after_run(h, h->plan_nvis)) != cudaSuccess) return cuda_fail(h, e, "cube fold");
         ++h->graph_launches;
@@ -539,7 +559,7 @@ extern "C" int vista_run(vista_stack *h)
     std::vector<SortLayout> layouts(classes.size());
     size_t sort_bytes = 0;
     int64_t rec_total = 0, cell_total = 0;
-    uint64_t nvis_run = 0;
+    uint64_t nvis_run = 0, bound_run = 0;
     std::vector<Copy2D> copies;
     std::vector<HostCopy> hcopies;
     std::vector<size_t> wave_pos((size_t)std::max(nwaves, 1), 0);   // next free byte of each wave's slot
@@ -643,6 +663,7 @@ extern "C" int vista_run(vista_stack *h)
                 for (const ChanF &f : pl.chf) nread += f.nb > 0;
                 for (int p = 0; p < s.d.npol; ++p) npm += s.pol_map[(size_t)p] >= 0;
                 nvis_run += (uint64_t)(d.nrow * nread * npm);
+                bound_run += entry_bound(s, pl);
             }
             roff[t + 1] = roff[t] + d.nrow;
             soff[t + 1] = soff[t] + (fp64 ? 0 : (d.nrow + SEG_ROWS - 1) / SEG_ROWS);
@@ -742,6 +763,7 @@ extern "C" int vista_run(vista_stack *h)
     for (const SrcHost &s : h->pending) any_host |= s.d.mem == VISTA_MEM_HOST;
     // host-memory windows: streamed wave by wave (their arrays must stay valid
     // until this stream work completes); otherwise the device pass at once
+    h->count_bound += bound_run;
     if ((e = (nwaves > 0 ? streamed_pass(h) : device_pass(h, h->stream))) != cudaSuccess) {
         h->plan_valid = false;
         return cuda_fail(h, e, "kernel launch or host-to-device copy");
@@ -758,6 +780,7 @@ extern "C" int vista_run(vista_stack *h)
     h->plan_valid = !any_host;
     h->plan_sig = run_signature(h);   // with the lattice as now fixed
     h->plan_nvis = nvis_run;
+    h->plan_bound = bound_run;
     h->last = std::move(h->pending);
     h->pending.clear();
     return VISTA_OK;
