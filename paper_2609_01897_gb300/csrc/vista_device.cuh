@@ -74,11 +74,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return false;
 }
 
-__device__ __forceinline__ float2 cmul(float2 a, float2 b)
-{
-    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
 // exp(2 pi i t) for a reduced turn count |t| <= 1/2 (|2 pi t| <= pi).
 // CUDA's __sincosf has an absolute error of at most 2^-21.41 on [-pi, pi]
 // (CUDA C Programming Guide, intrinsic functions), i.e. a phase error below
@@ -113,8 +108,8 @@ __device__ __host__ __forceinline__ void split_ff(double x, float &hi, float &lo
     lo = (float)(x - (double)hi);
 }
 
-// One axis of the uv cell: floor(fl64(coord * s_k)) + n/2, or -1 outside
-// [0, n).  Decided in FP32 when fl32(c32 * s32) is at least 2^-21 |x| away
+// The floor of one axis of the uv cell rule, floor(fl64(coord * s_k)),
+// decided in FP32 when fl32(c32 * s32) is at least 2^-21 |x| away
 // from an integer (the FP32 product differs from the FP64 one by at most
 // 3 * 2^-24 |x|), else by the exact FP64 product.
 // The exact FP64 product, out of line so that the compiler cannot hoist it
@@ -126,7 +121,7 @@ static __device__ __noinline__ float exact_floor_product(const double *coord64, 
     return (float)floor(__dmul_rn(c, *s64));
 }
 
-// floor(fl64(coord * s_k)) as a float (exact; see axis_cell).
+// floor(fl64(coord * s_k)) as a float (exact).
 __device__ __forceinline__ float axis_floor(float c32, float s32, const double *coord64, bool neg,
                                             const double *s64)
 {
@@ -136,15 +131,6 @@ __device__ __forceinline__ float axis_floor(float c32, float s32, const double *
     float fx = fa;
     if (__builtin_expect(fa != fb, 0)) fx = exact_floor_product(coord64, neg, s64);
     return fx;
-}
-
-__device__ __forceinline__ int axis_cell(float c32, float s32, const double *coord64, bool neg,
-                                         const double *s64, int n)
-{
-    const float fx = axis_floor(c32, s32, coord64, neg, s64);
-    float h = (float)(n >> 1);
-    if (!(fx >= -h && fx < h)) return -1;
-    return (int)fx + (n >> 1);
 }
 
 __device__ __forceinline__ int axis_cell64(double c, double s, int n)
@@ -195,106 +181,93 @@ __device__ __forceinline__ int chunk_cell_step(int2 cc, int kk, int nu)
     return c;
 }
 
-// ----------------------------------------------------------- vis loaders
+// ------------------------------------------------ stored visibility types
 
-template <int P, int VT>
-struct VisLoad;
-
-template <int P>
-struct VisLoad<P, VISTA_VIS_C64> {
-    static constexpr int kBytes = 8;   // bytes per complex value
-    static __device__ __forceinline__ void load(const void *base, int64_t idx, float scale, float2 (&v)[P])
+// Bytes of one complex value, and the 16-bit types' decoding.
+template <int VT>
+struct VisType {
+    static constexpr int kBytes = VT == VISTA_VIS_C128 ? 16 : VT == VISTA_VIS_C64 ? 8 : 4;
+    static __device__ __forceinline__ float2 half_pair(uint32_t b)
     {
-        (void)scale;
-        const float2 *p = reinterpret_cast<const float2 *>(base) + idx * P;
-        if constexpr (P == 1) {
-            v[0] = __ldcs(p);
-        } else if constexpr (P == 2) {
-            float4 q = __ldcs(reinterpret_cast<const float4 *>(p));
-            v[0] = make_float2(q.x, q.y);
-            v[1] = make_float2(q.z, q.w);
-        } else {
-            float4 q0 = __ldcs(reinterpret_cast<const float4 *>(p));
-            float4 q1 = __ldcs(reinterpret_cast<const float4 *>(p) + 1);
-            v[0] = make_float2(q0.x, q0.y);
-            v[1] = make_float2(q0.z, q0.w);
-            v[2] = make_float2(q1.x, q1.y);
-            v[3] = make_float2(q1.z, q1.w);
+        if constexpr (VT == VISTA_VIS_F16X2) {
+            return __half22float2(*reinterpret_cast<__half2 *>(&b));
+        } else {   // bf16 -> f32 is a 16-bit shift
+            return make_float2(__uint_as_float(b << 16), __uint_as_float(b & 0xffff0000u));
         }
     }
 };
 
+// ---- shared-memory loads at a 32-bit address plus a constant ----
+
+template <int OFF>
+__device__ __forceinline__ uint32_t lds32(uint32_t at)
+{
+    uint32_t x;
+    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(x) : "r"(at), "n"(OFF));
+    return x;
+}
+template <int OFF>
+__device__ __forceinline__ uint64_t lds64(uint32_t at)
+{
+    uint64_t x;
+    asm volatile("ld.shared.b64 %0, [%1+%2];" : "=l"(x) : "r"(at), "n"(OFF));
+    return x;
+}
+template <int OFF>
+__device__ __forceinline__ ulonglong2 lds128(uint32_t at)
+{
+    ulonglong2 x;
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2+%3];" : "=l"(x.x), "=l"(x.y) : "r"(at), "n"(OFF));
+    return x;
+}
+
+// ---- packed FP32 pairs (one instruction for both halves) ----
+
+__device__ __forceinline__ uint64_t pack2(float x, float y)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// A folded row's values conjugated (sign = the sign bit; 0 leaves them): with
+// its delay negated in the record, the shifted visibilities come out conjugated.
 template <int P>
-struct VisLoad<P, VISTA_VIS_C128> {
-    static constexpr int kBytes = 16;
-    static __device__ __forceinline__ void load(const void *base, int64_t idx, float scale, float2 (&v)[P])
-    {
-        (void)scale;
-        const double2 *p = reinterpret_cast<const double2 *>(base) + idx * P;
+__device__ __forceinline__ void conjugate(uint64_t (&v)[P], uint32_t sign)
+{
 #pragma unroll
-        for (int i = 0; i < P; ++i) {
-            double2 q = __ldcs(p + i);
-            v[i] = make_float2((float)q.x, (float)q.y);
-        }
-    }
-};
+    for (int p = 0; p < P; ++p) v[p] ^= (uint64_t)sign << 32;
+}
 
-
-template <int P>
-struct VisLoad<P, VISTA_VIS_F16X2> {
-    static constexpr int kBytes = 4;
-    static __device__ __forceinline__ float2 cvt(uint32_t b, float scale)
-    {
-        __half2 h = *reinterpret_cast<__half2 *>(&b);
-        float2 f = __half22float2(h);
-        return make_float2(f.x * scale, f.y * scale);
-    }
-    static __device__ __forceinline__ void load(const void *base, int64_t idx, float scale, float2 (&v)[P])
-    {
-        const uint32_t *p = reinterpret_cast<const uint32_t *>(base) + idx * P;
-        if constexpr (P == 1) {
-            v[0] = cvt(__ldcs(p), scale);
-        } else if constexpr (P == 2) {
-            uint2 q = __ldcs(reinterpret_cast<const uint2 *>(p));
-            v[0] = cvt(q.x, scale);
-            v[1] = cvt(q.y, scale);
-        } else {
-            uint4 q = __ldcs(reinterpret_cast<const uint4 *>(p));
-            v[0] = cvt(q.x, scale);
-            v[1] = cvt(q.y, scale);
-            v[2] = cvt(q.z, scale);
-            v[3] = cvt(q.w, scale);
-        }
-    }
-};
-
-template <int P>
-struct VisLoad<P, VISTA_VIS_BF16X2> {
-    static constexpr int kBytes = 4;
-    static __device__ __forceinline__ float2 cvt(uint32_t b, float scale)
-    {
-        // bf16 -> f32 is a 16-bit shift
-        float re = __uint_as_float(b << 16), im = __uint_as_float(b & 0xffff0000u);
-        return make_float2(re * scale, im * scale);
-    }
-    static __device__ __forceinline__ void load(const void *base, int64_t idx, float scale, float2 (&v)[P])
-    {
-        const uint32_t *p = reinterpret_cast<const uint32_t *>(base) + idx * P;
-        if constexpr (P == 1) {
-            v[0] = cvt(__ldcs(p), scale);
-        } else if constexpr (P == 2) {
-            uint2 q = __ldcs(reinterpret_cast<const uint2 *>(p));
-            v[0] = cvt(q.x, scale);
-            v[1] = cvt(q.y, scale);
-        } else {
-            uint4 q = __ldcs(reinterpret_cast<const uint4 *>(p));
-            v[0] = cvt(q.x, scale);
-            v[1] = cvt(q.y, scale);
-            v[2] = cvt(q.z, scale);
-            v[3] = cvt(q.w, scale);
-        }
-    }
-};
+// Adds one visibility V = (re, im), weighted WV = w V, to a lane's sums unless
+// its flag byte is set: C += w V c, S += w V s (as pairs; cc = (c, c), ss =
+// (s, s)), A += (w re^2, w im^2), sw += w, cnt += 1.  Predicated, so a flagged
+// value (whatever it holds) never enters.
+__device__ __forceinline__ void add_value(uint64_t &C, uint64_t &S, uint64_t &A, float &sw, uint32_t &cnt, uint64_t V,
+                                          uint64_t WV, float w, uint64_t cc, uint64_t ss, uint32_t flag)
+{
+    asm("{\n\t.reg .pred p;\n\t"
+        "setp.eq.u32 p, %11, 0;\n\t"
+        "@p fma.rn.f32x2 %0, %6, %8, %0;\n\t"
+        "@p fma.rn.f32x2 %1, %6, %9, %1;\n\t"
+        "@p fma.rn.f32x2 %2, %6, %5, %2;\n\t"
+        "@p add.rn.f32 %3, %3, %7;\n\t"
+        "@p add.u32 %4, %4, %10;\n\t}"
+        : "+l"(C), "+l"(S), "+l"(A), "+f"(sw), "+r"(cnt)
+        : "l"(V), "l"(WV), "f"(w), "l"(cc), "l"(ss), "n"(1), "r"(flag));
+}
 
 // ---- asynchronous copies of one lane's visibilities into shared memory ----
 
@@ -319,7 +292,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // 4-byte pieces and decoded from shared memory.
 template <int P, int VT>
 struct VisAsync {
-    static constexpr int kLaneBytes = P * VisLoad<P, VT>::kBytes;
+    static constexpr int kLaneBytes = P * VisType<VT>::kBytes;
     static __device__ __forceinline__ void copy(uint32_t dst, const void *src)
     {
         const char *s = reinterpret_cast<const char *>(src);
@@ -333,22 +306,77 @@ struct VisAsync {
             cp_async_4(dst, s);
         }
     }
-    static __device__ __forceinline__ void decode(const void *sm, float scale, float2 (&v)[P])
+    // The values at shared address at + OFF as (re, im) operand pairs.
+    template <int OFF>
+    static __device__ __forceinline__ void decode(uint32_t at, float scale, uint64_t (&v)[P])
     {
         if constexpr (VT == VISTA_VIS_C64) {
-            const float2 *q = reinterpret_cast<const float2 *>(sm);
-#pragma unroll
-            for (int i = 0; i < P; ++i) v[i] = q[i];
+            if constexpr (P == 1) {
+                v[0] = lds64<OFF>(at);
+            } else {
+                const ulonglong2 q = lds128<OFF>(at);
+                v[0] = q.x;
+                v[1] = q.y;
+                if constexpr (P == 4) {
+                    const ulonglong2 r = lds128<OFF + 16>(at);
+                    v[2] = r.x;
+                    v[3] = r.y;
+                }
+            }
         } else if constexpr (VT == VISTA_VIS_C128) {
-            const double2 *q = reinterpret_cast<const double2 *>(sm);
-#pragma unroll
-            for (int i = 0; i < P; ++i) v[i] = make_float2((float)q[i].x, (float)q[i].y);
+            auto one = [&](ulonglong2 q) {
+                return pack2((float)__longlong_as_double((long long)q.x), (float)__longlong_as_double((long long)q.y));
+            };
+            v[0] = one(lds128<OFF>(at));
+            if constexpr (P >= 2) v[1] = one(lds128<OFF + 16>(at));
+            if constexpr (P == 4) {
+                v[2] = one(lds128<OFF + 32>(at));
+                v[3] = one(lds128<OFF + 48>(at));
+            }
         } else {
-            const uint32_t *q = reinterpret_cast<const uint32_t *>(sm);
-#pragma unroll
-            for (int i = 0; i < P; ++i) v[i] = VisLoad<P, VT>::cvt(q[i], scale);
+            const uint64_t s2 = pack2(scale, scale);
+            auto one = [&](uint32_t b) {
+                const float2 f = VisType<VT>::half_pair(b);
+                return mul2(pack2(f.x, f.y), s2);
+            };
+            if constexpr (P == 1) {
+                v[0] = one(lds32<OFF>(at));
+            } else if constexpr (P == 2) {
+                const uint64_t q = lds64<OFF>(at);
+                v[0] = one((uint32_t)q);
+                v[1] = one((uint32_t)(q >> 32));
+            } else {
+                const ulonglong2 q = lds128<OFF>(at);
+                v[0] = one((uint32_t)q.x);
+                v[1] = one((uint32_t)(q.x >> 32));
+                v[2] = one((uint32_t)q.y);
+                v[3] = one((uint32_t)(q.y >> 32));
+            }
         }
     }
 };
+
+// P flag bytes (P-byte aligned) at shared address at + OFF, zero-extended.
+template <int P, int OFF>
+__device__ __forceinline__ uint32_t flag_bytes(uint32_t at)
+{
+    if constexpr (P == 4) {
+        return lds32<OFF>(at);
+    } else if constexpr (P == 2) {
+        uint16_t h;
+        asm volatile("ld.shared.u16 %0, [%1+%2];" : "=h"(h) : "r"(at), "n"(OFF));
+        return h;
+    } else {
+        uint32_t f;
+        asm volatile("ld.shared.u8 %0, [%1+%2];" : "=r"(f) : "r"(at), "n"(OFF));
+        return f;
+    }
+}
+
+// Vector reduction into one cube entry (no returned value).
+__device__ __forceinline__ void red_add4(void *p, float x, float y, float z, float w)
+{
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
 
 }  // namespace vista

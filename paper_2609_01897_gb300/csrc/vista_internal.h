@@ -119,15 +119,18 @@ static_assert(sizeof(SrcDev) % 16 == 0, "SrcDev is copied in 16-byte units");
 // Per-row record written by the mixed path's FP64 pre-pass (32 B), in
 // processing order.
 //   tau_hi + tau_lo  the delay tau (metres) as a float-float pair, so that
-//                    tau * nu_k / c is formed to ~1e-14 relative in FP32
-//   W[4]             the row's weights (>= 0), negated for a folded row: the
-//                    sign conjugates the shifted visibility, |W| is the weight
-//                    (the sign bit of W[0] marks the fold, also for W = 0)
+//                    tau * nu_k / c is formed to ~1e-14 relative in FP32;
+//                    negated for a folded row
 //   row              the row index in the window's arrays
+//   fold             the sign bit if the row is folded (its visibilities are
+//                    conjugated: with the negated delay the shifted
+//                    visibilities are too), else 0
+//   W[4]             the row's weights (>= 0); windows of 1 or 2 pols hold
+//                    each weight twice (W0 W0 W1 W1: operand pairs)
 struct __align__(16) RowRec {
     float tau_hi, tau_lo;
+    uint32_t row, fold;
     float W[4];
-    uint32_t row, pad;
 };
 static_assert(sizeof(RowRec) == 32, "RowRec is read as two 16-byte words");
 

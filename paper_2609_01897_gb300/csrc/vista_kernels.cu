@@ -26,14 +26,15 @@ __global__ void debug_mixed(RunArgs a, int src, double *ph_out, int32_t *cell_ou
     const RowRec rec = a.recs[S.rec_off + i];
     const int2 cc = a.ccells[S.cell_off + (int64_t)chunk * nrow + i];
     const int64_t row = rec.row;
-    const bool fold = signbit(rec.W[0]);
+    const bool fold = rec.fold != 0u;
 #pragma unroll
     for (int q = 0; q < NS; ++q) {
         const int kk = q * 32 + lane, k = c0 + kk;
         if (k < S.k_hi) {
             const ChanD *cd = a.chd + S.chan_off + (k - S.k_lo);
             const ChanF cf = a.chf[S.chan_off + (k - S.k_lo)];
-            const float2 ph = shift_phasor(rec.tau_hi, rec.tau_lo, cf.nuc_hi, cf.nuc_lo);
+            float2 ph = shift_phasor(rec.tau_hi, rec.tau_lo, cf.nuc_hi, cf.nuc_lo);
+            if (fold) ph.y = -ph.y;   // the record's delay is negated
             // same cell path as the stacking kernel
             int cid;
             if (cc.y == CC_NOCHANGE)

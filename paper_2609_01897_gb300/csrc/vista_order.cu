@@ -21,8 +21,7 @@
 //                  key (the rows of one key stay in row order), one
 //                  contiguous part of the bucket per warp
 //   k_rows         per row, in processing order: the FP64 delay of Eq. 2 as
-//                  a float-float pair, the (fold-signed) weights, and the
-//                  uv cells of each of the window's channel chunks
+//                  a float-float pair, the weights, and the uv cells of each of the window's channel chunks
 #include "vista_device.cuh"
 
 namespace vista {
@@ -477,7 +476,7 @@ __device__ int2 chunk_cell(const RunArgs &a, const SrcDev &S, const ChanF *cf, c
 }
 
 // One thread per row, in processing order: the row record (the FP64 delay
-// of Eq. 2 as a float-float pair, the fold-signed weights, the row index)
+// of Eq. 2 as a float-float pair, the weights, the row index)
 // and the chunk-cell entries of all the window's chunks, laid out
 // [chunk][row] per window so that an item's entries are contiguous.  The
 // row's coordinates are read once for both.  The window's channel table is
@@ -498,13 +497,13 @@ __global__ void __launch_bounds__(256) k_rows(RunArgs a)
     const double u = guvw[0], v = guvw[1];
     const bool fold = a.g.fold && (v < 0.0 || (v == 0.0 && u < 0.0));
     RowRec rec;
-    split_ff(tau, rec.tau_hi, rec.tau_lo);
+    split_ff(fold ? -tau : tau, rec.tau_hi, rec.tau_lo);
     rec.row = (uint32_t)r;
-    rec.pad = 0;
+    rec.fold = fold ? 0x80000000u : 0u;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float wk = k < S.npol ? S.wts[r * S.npol + k] : 0.0f;
-        rec.W[k] = fold ? -wk : wk;
+        const int p = S.npol == 4 ? k : k >> 1;
+        rec.W[k] = p < S.npol ? S.wts[r * S.npol + p] : 0.0f;
     }
     a.recs[S.rec_off + q] = rec;
 
