@@ -1,19 +1,30 @@
 // The paper's per-row output (Eq. 3): every row of one window regridded onto
 // the rest lattice, V_out(j) = sum_k V'(k) w_kj / sum_k w_kj over unflagged
 // channels, with V' the shifted visibility of Eq. 2 and w_kj the Eq. 4
-// weights.  The contributing channels of each output channel are listed on
-// the host (a compressed row table built from the FP64 planner's bins).  A
-// first kernel forms each row's delay in FP64 and keeps it as a float-float
-// pair; then one thread per (row, output channel) forms each contributor's
-// phasor as the stacking kernel does (float-float product tau nu_k / c,
-// reduced mod 1 turn, __sincosf: below 5e-7 rad) and sums in FP32 (a few
-// terms per output channel).  For complex64 with 2 or 4 pols on 16-byte
-// aligned arrays a channel's pols and their flags come in vector loads.
+// weights.
+//
+// k_regrid_prep forms, in FP64, each row's delay (kept as a float-float pair)
+// and each channel's rest bins and weights (the planner's rule, the same
+// rounded operations), and the range of channels that reach each output
+// channel.  k_regrid then gives every (output channel, pol) of a tile of R
+// rows a thread: its contributors' table entries are read once for R rows,
+// their R visibilities are independent loads, and the P threads of one output
+// channel compute R / P of the phasors each (as the stacking kernel does:
+// float-float product tau nu_k / c, reduced mod 1 turn, __sincosf, below 5e-7
+// rad) and exchange them by shuffles.  A warp's loads cover the pols of
+// neighbouring channels, so every 32-byte sector fetched is used whole (a
+// thread per (row, output channel) took 16 bytes of 32 different lines an
+// instruction and read the tables again for every row).  Bound by L1 lines a
+// load (wide windows, whose outputs' contributors lie several channels apart)
+// and by latency (narrow ones).  Kernel time, 12 000 rows x 3840 channels x 4
+// pols onto 1024: 437 -> 380 us (1.92 GB, 5.0 TB/s); 27 090 rows x 120
+// channels x 2 pols of FP16 onto 150: 87 -> 50 us.  Eight rows a tile: four
+// cost 6 % on the FP16 window, sixteen 10 % on the wide one; blocks of 128
+// columns 7 % on the wide one.  The tables were built on the host before
+// (130 and 50 us a call around the kernels, 65 and 40 us now).
+#include <climits>
 #include <cmath>
 #include <vector>
-
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
 
 #include "planner.h"
 #include "vista_device.cuh"
@@ -22,147 +33,240 @@
 namespace vista {
 namespace {
 
+// One channel as the regrid reads it (32 B).
+struct __align__(16) RegridChan {
+    int32_t j0, nb;         // rest bins j0 .. j0 + nb - 1 inside the lattice
+    float w[4];             // their Eq. 4 weights
+    float nuc_hi, nuc_lo;   // nu_k / c as a float-float pair (1/m)
+};
+
 struct RegridArgs {
     const double *uvw;
+    const double *freqs;    // [nchan]
     const void *vis;
     const uint8_t *flags;
-    const float2 *nuc;      // [nchan] nu_k / c as a float-float pair (1/m)
-    const int32_t *start;   // [nrest + 1] first contributor of each output channel
-    const int32_t *chan;    // contributing channel
-    const float *w;         // its Eq. 4 weight
+    RegridChan *chan;       // [nchan]
+    int32_t *range;         // [nrest][2] INT_MAX - first channel, last channel + 1 (zeros: none)
     float2 *tau;            // [nrow] the row's delay (m) as a float-float pair
     float *out_vis;         // [nrow][nrest][npol][2]
     float *out_wsum;        // [nrow][nrest][npol]
     double *out_uvw;        // [nrow][3] or null
     int64_t nrow;
-    int32_t nchan, npol, nrest, vis_type;
-    int32_t vec;            // complex64 with 2 or 4 pols, 16-byte aligned: a channel's pols in vector loads
-    int32_t vout;           // 2 or 4 pols, outputs 16-byte (wsum of 2 pols: 8-byte) aligned: vector stores
+    int32_t nchan, nrest, bin_mode;
+    uint32_t ncb;           // blocks of COLS columns a tile of rows takes
+    int32_t pair_out;       // out_vis is 8-byte aligned: a value's two floats in one store
     float vis_scale;
     double l, m, n1, inv_zf;
+    double zf, f0, df;      // 1 + z, the rest lattice
 };
 
-__device__ __forceinline__ float2 load_vis(const RegridArgs &a, int64_t i)
+// A channel's rest bins and weights: channel_bins() of the planner, operation
+// by operation.
+__device__ void rest_bins(const RegridArgs &a, int k, RegridChan &c)
 {
-    switch (a.vis_type) {
-    case VISTA_VIS_C128: {
-        const double2 v = reinterpret_cast<const double2 *>(a.vis)[i];
-        return make_float2((float)v.x, (float)v.y);
-    }
-    case VISTA_VIS_C64: return reinterpret_cast<const float2 *>(a.vis)[i];
-    case VISTA_VIS_F16X2: {
-        const __half2 v = reinterpret_cast<const __half2 *>(a.vis)[i];
-        return make_float2(__low2float(v) * a.vis_scale, __high2float(v) * a.vis_scale);
-    }
-    default: {
-        const __nv_bfloat162 v = reinterpret_cast<const __nv_bfloat162 *>(a.vis)[i];
-        return make_float2(__low2float(v) * a.vis_scale, __high2float(v) * a.vis_scale);
-    }
-    }
-}
-
-// One thread per row: the Eq. 2 delay in FP64, kept as a float-float pair,
-// and the rest-frame baseline (Eq. 1 with R = I) if asked for.
-__global__ void __launch_bounds__(256) k_regrid_tau(RegridArgs a)
-{
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= a.nrow) return;
-    const double *x = a.uvw + 3 * r;
-    float hi, lo;
-    split_ff(x[0] * a.l + x[1] * a.m + x[2] * a.n1, hi, lo);
-    a.tau[r] = make_float2(hi, lo);
-    if (a.out_uvw)
-        for (int c = 0; c < 3; ++c) a.out_uvw[3 * r + c] = x[c] * a.inv_zf;
-}
-
-// One channel's P visibilities (and their flag bytes, 0 = unflagged) with
-// vector loads: complex64 pols of a channel are 8 P contiguous, 16-byte
-// aligned bytes, their flags 4 (P = 4) or 2 (P = 2) aligned bytes.
-template <int P>
-__device__ __forceinline__ void load_channel_c64(const RegridArgs &a, int64_t i0, float2 (&v)[4], uint32_t &fl)
-{
-    const float4 *q = reinterpret_cast<const float4 *>(reinterpret_cast<const float2 *>(a.vis) + i0);
-    const float4 x = q[0];
-    v[0] = make_float2(x.x, x.y);
-    v[1] = make_float2(x.z, x.w);
-    if constexpr (P == 4) {
-        const float4 y = q[1];
-        v[2] = make_float2(y.x, y.y);
-        v[3] = make_float2(y.z, y.w);
-        fl = a.flags ? *reinterpret_cast<const uint32_t *>(a.flags + i0) : 0u;
-    } else {
-        fl = a.flags ? (uint32_t)*reinterpret_cast<const uint16_t *>(a.flags + i0) : 0u;
-    }
-}
-
-__global__ void __launch_bounds__(256) k_regrid(RegridArgs a)
-{
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= a.nrow * a.nrest) return;
-    const int64_t r = t / a.nrest;
-    const int j = (int)(t - r * a.nrest);
-    const float2 tau = a.tau[r];
-    float sr[4] = {0, 0, 0, 0}, si[4] = {0, 0, 0, 0}, sw[4] = {0, 0, 0, 0};
-    for (int e = a.start[j]; e < a.start[j + 1]; ++e) {
-        const int k = a.chan[e];
-        const float w = a.w[e];
-        const float2 nuc = a.nuc[k];
-        const float2 ph = shift_phasor(tau.x, tau.y, nuc.x, nuc.y);
-        const int64_t i0 = (r * a.nchan + k) * a.npol;
-        if (a.vec) {
-            float2 v[4];
-            uint32_t fl;
-            if (a.npol == 4) load_channel_c64<4>(a, i0, v, fl);
-            else load_channel_c64<2>(a, i0, v, fl);
-#pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                if (p >= a.npol || ((fl >> (8 * p)) & 0xffu)) continue;
-                sr[p] = __fmaf_rn(w, v[p].x * ph.x - v[p].y * ph.y, sr[p]);
-                si[p] = __fmaf_rn(w, v[p].x * ph.y + v[p].y * ph.x, si[p]);
-                sw[p] += w;
-            }
-            continue;
-        }
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            if (p >= a.npol) break;
-            const int64_t i = i0 + p;
-            if (a.flags && a.flags[i]) continue;
-            const float2 v = load_vis(a, i);
-            sr[p] = __fmaf_rn(w, v.x * ph.x - v.y * ph.y, sr[p]);
-            si[p] = __fmaf_rn(w, v.x * ph.y + v.y * ph.x, si[p]);
-            sw[p] += w;
-        }
-    }
-    float ov[8];
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const bool any = sw[p] > 0.0f;
-        ov[2 * p] = any ? sr[p] / sw[p] : 0.0f;
-        ov[2 * p + 1] = any ? si[p] / sw[p] : 0.0f;
-    }
-    const int64_t o = (r * a.nrest + j) * a.npol;
-    if (a.vout) {
-        // a thread's outputs are contiguous: whole 16-byte stores rather
-        // than one 4-byte store per value (each of those spans 32 sectors
-        // across the warp)
-        float4 *dv = reinterpret_cast<float4 *>(a.out_vis + 2 * o);
-        dv[0] = make_float4(ov[0], ov[1], ov[2], ov[3]);
-        if (a.npol == 4) {
-            dv[1] = make_float4(ov[4], ov[5], ov[6], ov[7]);
-            *reinterpret_cast<float4 *>(a.out_wsum + o) = make_float4(sw[0], sw[1], sw[2], sw[3]);
-        } else {
-            *reinterpret_cast<float2 *>(a.out_wsum + o) = make_float2(sw[0], sw[1]);
+    const double *f = a.freqs;
+    c.j0 = c.nb = 0;
+    c.w[0] = c.w[1] = c.w[2] = c.w[3] = 0.f;
+    if (a.bin_mode == VISTA_BIN_NEAREST) {
+        const double q = floor(__ddiv_rn(__dsub_rn(__dmul_rn(f[k], a.zf), a.f0), a.df));
+        if (q >= 0.0 && q < (double)a.nrest) {
+            c.j0 = (int32_t)q;
+            c.nb = 1;
+            c.w[0] = 1.f;
         }
         return;
     }
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        if (p >= a.npol) break;
-        a.out_vis[2 * (o + p)] = ov[2 * p];
-        a.out_vis[2 * (o + p) + 1] = ov[2 * p + 1];
-        a.out_wsum[o + p] = sw[p];
+    double d;
+    if (k == 0)
+        d = __dsub_rn(f[1], f[0]);
+    else if (k == a.nchan - 1)
+        d = __dsub_rn(f[k], f[k - 1]);
+    else
+        d = __dmul_rn(__dsub_rn(f[k + 1], f[k - 1]), 0.5);
+    const double half = __dmul_rn(0.5, fabs(d));
+    const double lo = __dmul_rn(__dsub_rn(f[k], half), a.zf), hi = __dmul_rn(__dadd_rn(f[k], half), a.zf);
+    double ca = floor(__ddiv_rn(__dsub_rn(lo, a.f0), a.df)) - 2.0, cb = floor(__ddiv_rn(__dsub_rn(hi, a.f0), a.df)) + 2.0;
+    if (ca < 0.0) ca = 0.0;
+    if (cb > (double)(a.nrest - 1)) cb = (double)(a.nrest - 1);
+    if (!(ca <= cb)) return;
+    int n = 0;
+    for (int64_t j = (int64_t)ca; j <= (int64_t)cb; ++j) {
+        const double e0 = __dadd_rn(a.f0, __dmul_rn((double)j, a.df));
+        const double e1 = __dadd_rn(a.f0, __dmul_rn((double)(j + 1), a.df));
+        const double o = __dsub_rn(hi < e1 ? hi : e1, lo > e0 ? lo : e0);
+        if (!(o > 0.0)) continue;
+        if (n == VISTA_MAX_BINS) break;   // (the host has refused such windows)
+        if (n == 0) c.j0 = (int32_t)j;
+        const float w = (float)__ddiv_rn(o, __dsub_rn(hi, lo));
+        if (n == 0) c.w[0] = w;
+        else if (n == 1) c.w[1] = w;
+        else if (n == 2) c.w[2] = w;
+        else c.w[3] = w;
+        ++n;
     }
+    c.nb = n;
+}
+
+// One thread per row and per channel: the Eq. 2 delay in FP64, kept as a
+// float-float pair, and the rest-frame baseline (Eq. 1 with R = I) if asked
+// for; the channel's table entry and its place in the ranges.
+__global__ void __launch_bounds__(128) k_regrid_prep(RegridArgs a)
+{
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < a.nrow) {
+        const double *x = a.uvw + 3 * r;
+        float hi, lo;
+        split_ff(x[0] * a.l + x[1] * a.m + x[2] * a.n1, hi, lo);
+        a.tau[r] = make_float2(hi, lo);
+        if (a.out_uvw)
+            for (int c = 0; c < 3; ++c) a.out_uvw[3 * r + c] = x[c] * a.inv_zf;
+    }
+    if (r < a.nchan) {
+        const int k = (int)r;
+        RegridChan c;
+        rest_bins(a, k, c);
+        const double nuc = __ddiv_rn(a.freqs[k], C_LIGHT);
+        split_ff(nuc, c.nuc_hi, c.nuc_lo);
+        a.chan[k] = c;
+        for (int b = 0; b < c.nb; ++b) {
+            atomicMax(a.range + 2 * (int64_t)(c.j0 + b), INT_MAX - k);
+            atomicMax(a.range + 2 * (int64_t)(c.j0 + b) + 1, k + 1);
+        }
+    }
+}
+
+// The visibility at `at`.
+template <int VT>
+__device__ __forceinline__ float2 load_value(const char *at, float scale)
+{
+    if constexpr (VT == VISTA_VIS_C128) {
+        const double2 v = __ldg(reinterpret_cast<const double2 *>(at));
+        return make_float2((float)v.x, (float)v.y);
+    } else if constexpr (VT == VISTA_VIS_C64) {
+        return __ldg(reinterpret_cast<const float2 *>(at));
+    } else {
+        const float2 v = VisType<VT>::half_pair(__ldg(reinterpret_cast<const uint32_t *>(at)));
+        return make_float2(v.x * scale, v.y * scale);
+    }
+}
+
+constexpr int COLS = 64;   // (output channel, pol) columns a block takes
+
+template <int P, int VT, int R>
+__global__ void __launch_bounds__(COLS, 14) k_regrid(RegridArgs a)
+{
+    constexpr int RP = R / P;   // rows whose phasors a thread computes
+    constexpr uint32_t VB = VisType<VT>::kBytes;
+    const int lane = threadIdx.x & 31, p = lane % P;
+    // the tile and its row pointers are the same for the whole block, so that
+    // a load's address is a uniform pointer plus the thread's 32-bit offset
+    const uint32_t tile = blockIdx.x / a.ncb;
+    const int64_t ncol = (int64_t)a.nrest * P, col = (int64_t)(blockIdx.x - tile * a.ncb) * COLS + threadIdx.x;
+    const bool in = col < ncol;   // (every lane takes part in the shuffles)
+    const int j = in ? (int)(col / P) : 0;
+    const int64_t r0 = (int64_t)tile * R;
+    const int nr = (int)(a.nrow - r0 < R ? a.nrow - r0 : R);
+    const int2 rg = in ? *reinterpret_cast<const int2 *>(a.range + 2 * (int64_t)j) : make_int2(0, 0);
+    const int first = INT_MAX - rg.x, cnt = rg.y > 0 ? rg.y - first : 0;
+    const int steps = __reduce_max_sync(0xffffffffu, cnt);
+    float2 tau[RP];   // rows p, p + P, ...
+#pragma unroll
+    for (int i = 0; i < RP; ++i) tau[i] = __ldg(a.tau + r0 + min(i * P + p, nr - 1));
+    float sr[R], si[R], sw[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) sr[r] = si[r] = sw[r] = 0.f;
+    const int64_t row_values = (int64_t)a.nchan * P;
+    const char *vis = reinterpret_cast<const char *>(a.vis) + r0 * row_values * VB;
+    const uint8_t *flags = a.flags ? a.flags + r0 * row_values : nullptr;
+    for (int e = 0; e < steps; ++e) {
+        const int k = first + e;
+        float w = 0.f, nh = 0.f, nl = 0.f;
+        if (e < cnt) {
+            const int4 c0 = __ldg(reinterpret_cast<const int4 *>(a.chan + k));        // j0, nb, w0, w1
+            const float4 c1 = __ldg(reinterpret_cast<const float4 *>(a.chan + k) + 1);   // w2, w3, nuc
+            const int b = j - c0.x;
+            if (b >= 0 && b < c0.y)
+                w = b == 0 ? __int_as_float(c0.z) : b == 1 ? __int_as_float(c0.w) : b == 2 ? c1.x : c1.y;
+            nh = c1.z;
+            nl = c1.w;
+        }
+        // the rows' values and flags, all in flight together (rows past the
+        // end re-read the last one, threads without a contributor channel 0)
+        const bool use = w > 0.f;
+        const uint32_t off = use ? (uint32_t)k * P + p : (uint32_t)p;
+        float2 v[R];
+        uint32_t fl[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = load_value<VT>(vis + min(r, nr - 1) * row_values * VB + off * VB, a.vis_scale);
+        if (flags) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) fl[r] = __ldg(flags + min(r, nr - 1) * row_values + off);
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) fl[r] = 0u;
+        }
+        float wc[RP], ws[RP];
+#pragma unroll
+        for (int i = 0; i < RP; ++i) {
+            const float2 ph = shift_phasor(tau[i].x, tau[i].y, nh, nl);
+            wc[i] = w * ph.x;
+            ws[i] = w * ph.y;
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float c = P == 1 ? wc[r / P] : __shfl_sync(0xffffffffu, wc[r / P], r % P, P);
+            const float s = P == 1 ? ws[r / P] : __shfl_sync(0xffffffffu, ws[r / P], r % P, P);
+            if (use && fl[r] == 0u) {
+                sr[r] = __fmaf_rn(v[r].x, c, __fmaf_rn(-v[r].y, s, sr[r]));
+                si[r] = __fmaf_rn(v[r].x, s, __fmaf_rn(v[r].y, c, si[r]));
+                sw[r] += w;
+            }
+        }
+    }
+    if (!in) return;
+    float2 *ov = reinterpret_cast<float2 *>(a.out_vis) + r0 * ncol + col;
+    float *ow = a.out_wsum + r0 * ncol + col;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (r >= nr) break;
+        const bool any = sw[r] > 0.0f;
+        const float re = any ? sr[r] / sw[r] : 0.0f, im = any ? si[r] / sw[r] : 0.0f;
+        if (a.pair_out) {
+            ov[r * ncol] = make_float2(re, im);
+        } else {
+            float *o = a.out_vis + 2 * ((r0 + r) * ncol + col);
+            o[0] = re;
+            o[1] = im;
+        }
+        ow[r * ncol] = sw[r];
+    }
+}
+
+// Rows a tile: eight where that leaves at least four warps of work per
+// scheduler (152 x 4 of them), else four.
+template <int P, int VT>
+cudaError_t launch_regrid_p(RegridArgs a, cudaStream_t st)
+{
+    const int64_t ncb = ((int64_t)a.nrest * P + COLS - 1) / COLS;
+    const bool eight = (a.nrow + 7) / 8 * ncb >= (int64_t)4 * 152;
+    const int R = eight ? 8 : 4;
+    const int64_t blocks = (a.nrow + R - 1) / R * ncb;
+    // a tile's values lie within 32-bit offsets of its row pointers
+    if (blocks > (int64_t)INT_MAX || (int64_t)a.nchan * P * VisType<VT>::kBytes > (int64_t)UINT32_MAX)
+        return cudaErrorInvalidValue;
+    a.ncb = (uint32_t)ncb;
+    if (eight)
+        k_regrid<P, VT, 8><<<(unsigned)blocks, COLS, 0, st>>>(a);
+    else
+        k_regrid<P, VT, 4><<<(unsigned)blocks, COLS, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int VT>
+cudaError_t launch_regrid_vt(const RegridArgs &a, int npol, cudaStream_t st)
+{
+    return npol == 4 ? launch_regrid_p<4, VT>(a, st) : npol == 2 ? launch_regrid_p<2, VT>(a, st)
+                                                                : launch_regrid_p<1, VT>(a, st);
 }
 
 }  // namespace
@@ -197,82 +301,63 @@ extern "C" int vista_regrid_rows(vista_stack *h, const vista_source_desc *s, flo
             return fail(h, VISTA_E_ARG, "freqs must be strictly monotone (index %d)", k);
     if (s->nrow == 0) return VISTA_OK;
 
-    // contributors of each output channel (Eq. 4), from the FP64 planner
-    std::vector<int32_t> j0((size_t)n), nb((size_t)n);
-    std::vector<double> wk((size_t)n * VISTA_MAX_BINS);
-    const int rc = channel_bins(s->freqs, n, s->z, h->f0, h->df, nrest, h->desc.bin_mode, j0.data(), nb.data(),
-                                wk.data());
-    if (rc != VISTA_OK) return fail(h, rc, "channel planning failed");
-    std::vector<int32_t> start((size_t)nrest + 1, 0);
-    for (int32_t k = 0; k < n; ++k)
-        for (int b = 0; b < nb[(size_t)k]; ++b) ++start[(size_t)j0[(size_t)k] + b + 1];
-    for (int32_t j = 0; j < nrest; ++j) start[(size_t)j + 1] += start[(size_t)j];
-    const size_t nnz = (size_t)start[(size_t)nrest];
-    std::vector<int32_t> chan(nnz > 0 ? nnz : 1), fill(start.begin(), start.end() - 1);
-    std::vector<float> w(nnz > 0 ? nnz : 1);
-    for (int32_t k = 0; k < n; ++k)
-        for (int b = 0; b < nb[(size_t)k]; ++b) {
-            const int32_t e = fill[(size_t)j0[(size_t)k] + b]++;
-            chan[(size_t)e] = k;
-            w[(size_t)e] = (float)wk[(size_t)k * VISTA_MAX_BINS + b];
-        }
-
-    // nu_k / c of every channel as a float-float pair
-    std::vector<float2> nuc((size_t)n);
-    for (int32_t k = 0; k < n; ++k) {
-        const double x = s->freqs[k] / C_LIGHT;
-        nuc[(size_t)k].x = (float)x;
-        nuc[(size_t)k].y = (float)(x - (double)nuc[(size_t)k].x);
+    // a channel that may reach more than VISTA_MAX_BINS rest bins (wider than
+    // VISTA_MAX_BINS - 1 of them): the planner's own count decides
+    if (h->desc.bin_mode == VISTA_BIN_OVERLAP &&
+        !(widest_rest_channel(s->freqs, n, s->z) <= (VISTA_MAX_BINS - 1.001) * h->df)) {
+        std::vector<int32_t> j0((size_t)n), nb((size_t)n);
+        std::vector<double> wk((size_t)n * VISTA_MAX_BINS);
+        const int rc = channel_bins(s->freqs, n, s->z, h->f0, h->df, nrest, h->desc.bin_mode, j0.data(), nb.data(),
+                                    wk.data());
+        if (rc != VISTA_OK) return fail(h, rc, "channel planning failed");
     }
 
-    // one device buffer: nu/c | start | chan | w | per-row delays
+    // one device buffer: frequencies | channel table | ranges | per-row delays
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    const size_t o_f = 0, o_s = al(sizeof(float2) * (size_t)n), o_c = o_s + al(sizeof(int32_t) * start.size()),
-                 o_w = o_c + al(sizeof(int32_t) * chan.size()), o_t = o_w + al(sizeof(float) * w.size()),
-                 total = o_t + al(sizeof(float2) * (size_t)s->nrow);
+    const size_t o_c = al(sizeof(double) * (size_t)n), o_r = o_c + al(sizeof(RegridChan) * (size_t)n),
+                 o_t = o_r + al(sizeof(int32_t) * 2 * (size_t)nrest), total = o_t + al(sizeof(float2) * (size_t)s->nrow);
     cudaError_t e = h->b_regrid.ensure(total);
     if (e != cudaSuccess) return cuda_fail(h, e, "regrid table allocation");
     char *b = (char *)h->b_regrid.p;
-    e = cudaMemcpyAsync(b + o_f, nuc.data(), sizeof(float2) * (size_t)n, cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b + o_s, start.data(), sizeof(int32_t) * start.size(), cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b + o_c, chan.data(), sizeof(int32_t) * chan.size(), cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b + o_w, w.data(), sizeof(float) * w.size(), cudaMemcpyHostToDevice, h->stream);
+    e = cudaMemcpyAsync(b, s->freqs, sizeof(double) * (size_t)n, cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b + o_r, 0, sizeof(int32_t) * 2 * (size_t)nrest, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "regrid table upload");
 
     RegridArgs a{};
     a.uvw = s->uvw;
+    a.freqs = (const double *)b;
     a.vis = s->vis;
     a.flags = s->flags;
-    a.nuc = (const float2 *)(b + o_f);
-    a.start = (const int32_t *)(b + o_s);
-    a.chan = (const int32_t *)(b + o_c);
-    a.w = (const float *)(b + o_w);
+    a.chan = (RegridChan *)(b + o_c);
+    a.range = (int32_t *)(b + o_r);
     a.tau = (float2 *)(b + o_t);
     a.out_vis = out_vis;
     a.out_wsum = out_wsum;
     a.out_uvw = out_uvw;
     a.nrow = s->nrow;
     a.nchan = n;
-    a.npol = s->npol;
     a.nrest = nrest;
-    a.vis_type = s->vis_type;
+    a.bin_mode = h->desc.bin_mode;
+    a.pair_out = ((uintptr_t)out_vis % 8) == 0;
     a.vis_scale = (s->vis_type == VISTA_VIS_F16X2 || s->vis_type == VISTA_VIS_BF16X2) ? s->vis_scale : 1.0f;
-    a.vec = s->vis_type == VISTA_VIS_C64 && (s->npol == 2 || s->npol == 4) && ((uintptr_t)s->vis % 16) == 0 &&
-            (!s->flags || ((uintptr_t)s->flags % (uintptr_t)s->npol) == 0);
-    a.vout = (s->npol == 2 || s->npol == 4) && ((uintptr_t)out_vis % 16) == 0 &&
-             ((uintptr_t)out_wsum % (uintptr_t)(s->npol == 4 ? 16 : 8)) == 0;
+    a.zf = 1.0 + s->z;
+    a.f0 = h->f0;
+    a.df = h->df;
     a.l = s->l;
     a.m = s->m;
     a.n1 = std::sqrt(1.0 - s->l * s->l - s->m * s->m) - 1.0;
     a.inv_zf = 1.0 / (1.0 + s->z);
-    const int64_t threads = s->nrow * (int64_t)nrest;
-    k_regrid_tau<<<(unsigned)((s->nrow + 255) / 256), 256, 0, h->stream>>>(a);
+    const int64_t prep = s->nrow > n ? s->nrow : n;
+    k_regrid_prep<<<(unsigned)((prep + 127) / 128), 128, 0, h->stream>>>(a);
     e = cudaGetLastError();
-    if (e == cudaSuccess) k_regrid<<<(unsigned)((threads + 255) / 256), 256, 0, h->stream>>>(a);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) {
+        switch (s->vis_type) {
+        case VISTA_VIS_C64: e = launch_regrid_vt<VISTA_VIS_C64>(a, s->npol, h->stream); break;
+        case VISTA_VIS_C128: e = launch_regrid_vt<VISTA_VIS_C128>(a, s->npol, h->stream); break;
+        case VISTA_VIS_F16X2: e = launch_regrid_vt<VISTA_VIS_F16X2>(a, s->npol, h->stream); break;
+        default: e = launch_regrid_vt<VISTA_VIS_BF16X2>(a, s->npol, h->stream); break;
+        }
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "regrid kernel");
     return VISTA_OK;
