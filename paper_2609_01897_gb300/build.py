@@ -21,7 +21,7 @@ LIB = os.path.join(HERE, "libvista.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["vista_stack_c64.cu", "vista_stack_c128.cu", "vista_stack_f16.cu", "vista_stack_bf16.cu",
-              "vista_stack.cu", "vista_kernels.cu", "vista_order.cu", "vista_run.cu", "vista_api.cu", "vista_regrid.cu",
+              "vista_stack.cu", "vista_fp64.cu", "vista_kernels.cu", "vista_order.cu", "vista_run.cu", "vista_api.cu", "vista_regrid.cu",
               "vista_noalloc.cu", "vista_autotune.cu", "vista_contsub.cu"]
 CXX_SOURCES = ["planner.cpp"]
 

@@ -102,7 +102,7 @@ struct SrcDev {
     int32_t nchunk;         // work chunks along the channel axis
     int32_t vstride;        // channels per stored row (nchan, or k_hi - k_lo when staged)
     int32_t kbase;          // channel index of the first stored channel
-    int32_t rot1;           // 1 + index of the window's R in RunArgs::rot (k_rotate fills guvw), 0 = none
+    int32_t rot1;           // 1 + index of the window's R in RunArgs::rot (k_keys fills guvw), 0 = none
     float key_su, key_sv;   // fl32(s_k) at the row-ordering reference channel
     int64_t rec_off;        // first row record of this window
     int64_t cell_off;       // first chunk-cell entry of this window ([chunk][row] inside)
@@ -201,7 +201,7 @@ struct SortArgs {
     int32_t rows_per_item;
 };
 
-// Everything one mixed or FP64 launch class needs on the device.
+// Everything one launch class needs on the device.
 struct RunArgs {
     const SrcDev *srcs;
     int32_t nsrc;
@@ -230,10 +230,8 @@ cudaError_t launch_prepare(const RunArgs &a, cudaStream_t st, int *nlaunch = nul
 // Persistent stacking kernel of one mixed class; key = (vis_type << 16) |
 // (chans_per_lane << 8) | npol, shared by every window of the class.
 cudaError_t launch_mixed(const RunArgs &a, int key, int warps_per_cta, int prefetch, cudaStream_t st);
-cudaError_t launch_fp64(const RunArgs &a, cudaStream_t st);
-// The gridding baselines R (u, v, w) of the class's re-projected windows
-// (a.rot non-null; one thread per row of the class), for the FP64 form.
-cudaError_t launch_rotate(const RunArgs &a, cudaStream_t st);
+// The FP64 stacking kernel of one class (chunks of 32 channels), same key.
+cudaError_t launch_fp64(const RunArgs &a, int key, cudaStream_t st);
 // Mixed cube: move every FP32 partial into the FP64 master and clear it.
 cudaError_t launch_fold(void *cube, double *master, int64_t n, cudaStream_t st);
 // Cube -> caller arrays; all = 1 reads every entry's sums, also where its count is 0.

@@ -1,10 +1,11 @@
-// libvista stacking kernels for sm_103a.
+// libvista kernels over the cube, for sm_103a.
 //
-//   (the mixed-precision stacking kernel is in vista_stack.cu)
-//   stack_fp64    the plain form: thread per (window, row), FP64 phasor
-//                 recurrence, FP64 cells, FP64 atomics into an FP64 cube
-//   debug_mixed   the mixed path's own phasor and cell code, exported
+//   (the stacking kernels are in vista_stack.cuh and vista_fp64.cu)
+//   debug_*       the phasors and cells of the two forms, exported
 //   unpack        cube -> caller arrays
+//   zero          the touched entries back to zero
+//   sparse_*      the touched entries -> caller arrays
+//   fold          FP32 partials -> FP64 master
 #include "vista_cube.cuh"
 #include "vista_device.cuh"
 
@@ -58,127 +59,40 @@ __global__ void debug_mixed(RunArgs a, int src, double *ph_out, int32_t *cell_ou
     }
 }
 
-// ------------------------------------------------------------- stack_fp64
-
-__device__ __forceinline__ double2 turns_to_phasor64(double t)
+// Debug export of the FP64 form's phasors and cells: the FP64 phase of every
+// channel that reaches the cube (the stacking kernel's recurrence is seeded
+// from the same expression at each chunk of 32 channels) and the FP64 cell
+// rule, one thread per row.
+__global__ void __launch_bounds__(128) debug_fp64(RunArgs a, int src, double *ph_out, int32_t *cell_out)
 {
-    double s, c;
-    sincospi(2.0 * t, &s, &c);
-    return make_double2(c, s);
-}
-
-__device__ __forceinline__ double2 cmul64(double2 a, double2 b)
-{
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
-template <bool EXPORT>
-__global__ void __launch_bounds__(128) stack_fp64(RunArgs a, int only_src, double *ph_out, int32_t *cell_out)
-{
-    const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= a.nrows_total) return;
-    const int s = find_owner(a.row_off, a.nsrc, gid);
-    if (EXPORT && s != only_src) return;
-    const SrcDev &S = a.srcs[s];
-    const int64_t r = gid - a.row_off[s];
+    const SrcDev &S = a.srcs[src];
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= S.nrow) return;
     const double *uvw = S.uvw + 3 * r;     // the stored baseline: the delay of Eq. 2
     const double tau = uvw[0] * S.l + uvw[1] * S.m + uvw[2] * S.n1;
     double u = S.guvw[3 * r], v = S.guvw[3 * r + 1];   // the gridding baseline (Eq. 1)
-    const bool fold = a.g.fold && (v < 0.0 || (v == 0.0 && u < 0.0));
-    if (fold) {
+    if (a.g.fold && (v < 0.0 || (v == 0.0 && u < 0.0))) {
         u = -u;
         v = -v;
     }
-    const int npol = S.npol, nrest = a.g.nrest, npol_c = a.g.npol;
-    double W[4];
-    for (int p = 0; p < 4; ++p) W[p] = p < npol ? (double)S.wts[r * npol + p] : 0.0;
     const ChanD *cd = a.chd + S.chan_off;
-    double2 ph = make_double2(1.0, 0.0), stp = make_double2(1.0, 0.0);
-    if (S.linear && S.k_hi > S.k_lo) {
-        const double t = tau * (cd[0].nu * (1.0 / C_LIGHT));
-        ph = turns_to_phasor64(t - floor(t));
-        const double d = tau * S.step_c;
-        stp = turns_to_phasor64(d - floor(d));
-    }
-    double *cube = reinterpret_cast<double *>(a.cube);
-    unsigned long long n_vis = 0, n_flag = 0, n_duv = 0, n_stk = 0;
     for (int k = S.k_lo; k < S.k_hi; ++k) {
-        const ChanD c = cd[k - S.k_lo];
-        if (!S.linear) {
+        const ChanD &c = cd[k - S.k_lo];
+        if (c.nb <= 0) continue;
+        const int64_t o = r * S.nchan + k;
+        if (ph_out) {
             const double t = tau * (c.nu * (1.0 / C_LIGHT));
-            ph = turns_to_phasor64(t - floor(t));
+            double s, co;
+            sincospi(2.0 * (t - floor(t)), &s, &co);
+            ph_out[2 * o] = co;
+            ph_out[2 * o + 1] = s;
         }
-        if (c.nb > 0) {
-            const int iu = axis_cell64(u, c.su, a.g.nu);
-            const int iv = axis_cell64(v, c.sv, a.g.nv);
-            const bool inuv = iu >= 0 && iv >= 0;
-            if (EXPORT) {
-                const int64_t o = r * S.nchan + k;
-                if (ph_out) {
-                    ph_out[2 * o] = ph.x;
-                    ph_out[2 * o + 1] = ph.y;
-                }
-                if (cell_out) {
-                    cell_out[2 * o] = inuv ? iu : -1;
-                    cell_out[2 * o + 1] = inuv ? iv : -1;
-                }
-            } else {
-                const int64_t vi = (r * S.vstride + (k - S.kbase)) * npol;
-                for (int p = 0; p < npol; ++p) {
-                    const int q = S.plane[p];
-                    if (q < 0) continue;
-                    ++n_vis;
-                    if (S.fbase && S.fbase[r * S.fpitch + (int64_t)(k - S.fk0) * npol + p]) {
-                        ++n_flag;
-                        continue;
-                    }
-                    if (!inuv) {
-                        ++n_duv;
-                        continue;
-                    }
-                    ++n_stk;
-                    double vr, vim;
-                    if (S.vis_type == VISTA_VIS_C128) {
-                        const double2 z2 = reinterpret_cast<const double2 *>(S.vis)[vi + p];
-                        vr = z2.x;
-                        vim = z2.y;
-                    } else if (S.vis_type == VISTA_VIS_C64) {
-                        const float2 z2 = reinterpret_cast<const float2 *>(S.vis)[vi + p];
-                        vr = z2.x;
-                        vim = z2.y;
-                    } else if (S.vis_type == VISTA_VIS_F16X2) {
-                        const __half2 h = reinterpret_cast<const __half2 *>(S.vis)[vi + p];
-                        vr = (double)__low2float(h) * (double)S.vis_scale;
-                        vim = (double)__high2float(h) * (double)S.vis_scale;
-                    } else {
-                        const __nv_bfloat162 h = reinterpret_cast<const __nv_bfloat162 *>(S.vis)[vi + p];
-                        vr = (double)__low2float(h) * (double)S.vis_scale;
-                        vim = (double)__high2float(h) * (double)S.vis_scale;
-                    }
-                    const double sr = vr * ph.x - vim * ph.y;
-                    double si = vr * ph.y + vim * ph.x;
-                    if (fold) si = -si;
-                    const double a2 = vr * vr + vim * vim;
-                    const size_t base = (((size_t)(iv * a.g.nu + iu) * nrest + c.j0) * npol_c + q);
-                    for (int b = 0; b < c.nb; ++b) {
-                        const double ww = W[p] * c.w[b];
-                        double *e = cube + 4 * (base + (size_t)b * npol_c);
-                        atomicAdd(e + 0, ww * sr);
-                        atomicAdd(e + 1, ww * si);
-                        atomicAdd(e + 2, ww);
-                        atomicAdd(e + 3, ww * a2);
-                        atomicAdd(a.count + base + (size_t)b * npol_c, 1u);
-                    }
-                }
-            }
+        if (cell_out) {
+            const int iu = axis_cell64(u, c.su, a.g.nu), iv = axis_cell64(v, c.sv, a.g.nv);
+            const bool on = iu >= 0 && iv >= 0;
+            cell_out[2 * o] = on ? iu : -1;
+            cell_out[2 * o + 1] = on ? iv : -1;
         }
-        if (S.linear) ph = cmul64(ph, stp);
-    }
-    if (!EXPORT) {
-        if (n_vis) atomicAdd(&a.stats->n_vis, n_vis);
-        if (n_flag) atomicAdd(&a.stats->n_flagged, n_flag);
-        if (n_duv) atomicAdd(&a.stats->n_dropped_uv, n_duv);
-        if (n_stk) atomicAdd(&a.stats->n_stacked, n_stk);
     }
 }
 
@@ -409,14 +323,6 @@ __global__ void __launch_bounds__(SPARSE_THREADS) sparse_write_kernel(const void
 
 // --------------------------------------------------------------- launchers
 
-cudaError_t launch_fp64(const RunArgs &a, cudaStream_t st)
-{
-    if (a.nrows_total == 0) return cudaSuccess;
-    const int64_t blocks = (a.nrows_total + 127) / 128;
-    stack_fp64<false><<<(unsigned)blocks, 128, 0, st>>>(a, -1, nullptr, nullptr);
-    return cudaGetLastError();
-}
-
 // ------------------------------------------------------------------ fold
 
 // Every nonzero FP32 entry of the mixed cube is added to its FP64 master
@@ -500,17 +406,15 @@ cudaError_t launch_sparse_write(const void *cube, const double *master, const ui
 
 cudaError_t launch_debug(const RunArgs &a, int ns, int src, int fp64, double *ph, int32_t *cells, cudaStream_t st)
 {
-    if (fp64) {
-        if (a.nrows_total == 0) return cudaSuccess;
-        const int64_t blocks = (a.nrows_total + 127) / 128;
-        stack_fp64<true><<<(unsigned)blocks, 128, 0, st>>>(a, src, ph, cells);
-        return cudaGetLastError();
-    }
     SrcDev S;
     cudaError_t e = cudaMemcpyAsync(&S, a.srcs + src, sizeof(S), cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return e;
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
+    if (fp64) {
+        if (S.nrow > 0) debug_fp64<<<(unsigned)((S.nrow + 127) / 128), 128, 0, st>>>(a, src, ph, cells);
+        return cudaGetLastError();
+    }
     const int64_t tasks = S.nrow * S.nchunk;
     if (tasks == 0) return cudaSuccess;
     const int64_t blocks = (tasks + 3) / 4;

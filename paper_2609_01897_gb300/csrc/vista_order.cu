@@ -521,27 +521,6 @@ __global__ void __launch_bounds__(256) k_rows(RunArgs a)
     }
 }
 
-// Re-projected windows (Eq. 1): their gridding baselines R (u, v, w) (see
-// rotate_row), one thread per row.  The mixed path forms them in k_keys,
-// which reads every row anyway; this kernel serves the plain FP64 form.
-__global__ void __launch_bounds__(256) k_rotate(RunArgs a)
-{
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.nrows_total) return;
-    const int w = find_owner(a.row_off, a.nsrc, p);
-    const SrcDev &S = a.srcs[w];
-    if (!S.rot1) return;
-    const int64_t r = p - a.row_off[w];
-    rotate_row(a.rot + 9 * (int64_t)(S.rot1 - 1), S.uvw + 3 * r, const_cast<double *>(S.guvw) + 3 * r);
-}
-
-cudaError_t launch_rotate(const RunArgs &a, cudaStream_t st)
-{
-    if (!a.rot || a.nrows_total == 0) return cudaSuccess;
-    k_rotate<<<(unsigned)((a.nrows_total + 255) / 256), 256, 0, st>>>(a);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_prepare(const RunArgs &a, cudaStream_t st, int *nlaunch)
 {
     const SortArgs &so = a.so;

@@ -10,8 +10,8 @@
 //      streams) run while the wave before is stacked, two staging slots
 //      taking turns (the streaming pipeline of Sec. 3.1/3.3: read ->
 //      compute overlapped)
-//   5. per mixed class: row ordering + records + work list, then the
-//      persistent stacking kernel; FP64 precision: the plain kernel
+//   5. per class: row ordering + records + work list, then the persistent
+//      stacking kernel (mixed or FP64)
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -210,8 +210,7 @@ SortLayout sort_layout(int64_t rows, int64_t nbuckets, int64_t max_items, int64_
     return L;
 }
 
-// One launch class: the row-ordering pre-pass and the stacking kernel (or
-// the FP64 kernel).
+// One launch class: the row-ordering pre-pass and the stacking kernel.
 cudaError_t launch_class(vista_stack *h, const ClassRun &cr, cudaStream_t st)
 {
     const bool fp64 = h->desc.precision == VISTA_PREC_FP64;
@@ -219,32 +218,16 @@ cudaError_t launch_class(vista_stack *h, const ClassRun &cr, cudaStream_t st)
     cudaError_t e = cudaSuccess;
     {
         const RunArgs &a = cr.args;
-        if (a.rot && fp64) {
-            // gridding baselines of the re-projected windows (the mixed path
-            // forms them in its pre-pass)
-            const int sp = span_begin(h, 0);
-            e = launch_rotate(a, st);
+        int sp = span_begin(h, 0);
+        int nk = 0;
+        e = launch_prepare(a, st, &nk);
+        span_end(h, sp);
+        if (h->timing) h->tacc.launches += nk;
+        if (e == cudaSuccess) {
+            sp = span_begin(h, 1);
+            e = fp64 ? launch_fp64(a, cr.key, st) : launch_mixed(a, cr.key, cfg.warps_per_cta, cfg.prefetch_rows, st);
             span_end(h, sp);
             if (h->timing) h->tacc.launches += 1;
-            if (e != cudaSuccess) return e;
-        }
-        if (fp64) {
-            const int sp = span_begin(h, 1);
-            e = launch_fp64(a, st);
-            span_end(h, sp);
-            if (h->timing) h->tacc.launches += 1;
-        } else {
-            int sp = span_begin(h, 0);
-            int nk = 0;
-            e = launch_prepare(a, st, &nk);
-            span_end(h, sp);
-            if (h->timing) h->tacc.launches += nk;
-            if (e == cudaSuccess) {
-                sp = span_begin(h, 1);
-                e = launch_mixed(a, cr.key, cfg.warps_per_cta, cfg.prefetch_rows, st);
-                span_end(h, sp);
-                if (h->timing) h->tacc.launches += 1;
-            }
         }
     }
     return e;
@@ -498,7 +481,7 @@ extern "C" int vista_run(vista_stack *h)
         const int cap = s.d.npol == 4 ? std::min(2, (int)cfg.chans_per_lane) : (int)cfg.chans_per_lane;
         const int ns = fp64 ? 1 : choose_ns(pl.k_hi - pl.k_lo, cap);
         ns_of[(size_t)i] = ns;
-        const int key = fp64 ? 0 : ((s.d.vis_type << 16) | (ns << 8) | s.d.npol);
+        const int key = (s.d.vis_type << 16) | (ns << 8) | s.d.npol;
         const int wv = wave_of[(size_t)i];
         int ci = -1;
         for (size_t j = 0; j < classes.size(); ++j)
@@ -548,7 +531,7 @@ extern "C" int vista_run(vista_stack *h)
     std::vector<SrcDev> sdev;
     std::vector<double> rots;   // 9 per re-projected window (SrcDev::rot1 - 1 indexes them)
     std::vector<char> cls_rot(classes.size(), 0);
-    // gridding baselines of the re-projected windows (filled by k_rotate)
+    // gridding baselines of the re-projected windows (filled by k_keys)
     int64_t rot_rows = 0, guvw_pos = 0;
     for (const SrcHost &s : h->pending)
         if (s.has_rot) rot_rows += s.d.nrow;
@@ -654,10 +637,8 @@ extern "C" int vista_run(vista_stack *h)
             d.key_sv = (float)(s.freqs[(size_t)pl.key_ch] * gv);
             d.rec_off = rec_total;
             d.cell_off = cell_total;
-            if (!fp64) {
-                rec_total += d.nrow;
-                cell_total += d.nrow * d.nchunk;
-            }
+            rec_total += d.nrow;
+            cell_total += d.nrow * d.nchunk;
             {
                 int64_t nread = 0, npm = 0;
                 for (const ChanF &f : pl.chf) nread += f.nb > 0;
@@ -666,7 +647,7 @@ extern "C" int vista_run(vista_stack *h)
                 bound_run += entry_bound(s, pl);
             }
             roff[t + 1] = roff[t] + d.nrow;
-            soff[t + 1] = soff[t] + (fp64 ? 0 : (d.nrow + SEG_ROWS - 1) / SEG_ROWS);
+            soff[t + 1] = soff[t] + (d.nrow + SEG_ROWS - 1) / SEG_ROWS;
             max_items += (int64_t)d.nchunk * ((d.nrow + cfg.rows_per_item - 1) / cfg.rows_per_item + h->nstripe);
             d.guvw = d.uvw;
             if (s.has_rot) {
@@ -702,16 +683,14 @@ extern "C" int vista_run(vista_stack *h)
     if (!rots.empty() && (e = up.put(h->b_rot, rots)) != cudaSuccess)
         return cuda_fail(h, e, "re-projection table upload");
     if ((e = up.end()) != cudaSuccess) return cuda_fail(h, e, "pinned staging of the tables");
-    if (!fp64) {
-        if ((e = h->b_recs.ensure((size_t)(rec_total > 0 ? rec_total : 1) * sizeof(RowRec))) != cudaSuccess)
-            return cuda_fail(h, e, "row record allocation");
-        // padding: the bulk copy of an item's chunk cells starts and ends on
-        // 16-byte boundaries, up to one entry past the last
-        if ((e = h->b_cells.ensure((size_t)(cell_total + 4) * sizeof(int2))) != cudaSuccess)
-            return cuda_fail(h, e, "chunk cell allocation");
-        if ((e = h->b_sort.ensure(sort_bytes > 0 ? sort_bytes : 256)) != cudaSuccess)
-            return cuda_fail(h, e, "ordering buffer allocation");
-    }
+    if ((e = h->b_recs.ensure((size_t)(rec_total > 0 ? rec_total : 1) * sizeof(RowRec))) != cudaSuccess)
+        return cuda_fail(h, e, "row record allocation");
+    // padding: the bulk copy of an item's chunk cells starts and ends on
+    // 16-byte boundaries, up to one entry past the last
+    if ((e = h->b_cells.ensure((size_t)(cell_total + 4) * sizeof(int2))) != cudaSuccess)
+        return cuda_fail(h, e, "chunk cell allocation");
+    if ((e = h->b_sort.ensure(sort_bytes > 0 ? sort_bytes : 256)) != cudaSuccess)
+        return cuda_fail(h, e, "ordering buffer allocation");
 
     // 5. launch arguments, then the device pass
     const CubeGeom g{c.nu, c.nv, c.nrest, c.npol, gu, gv, c.hermitian_fold, 0};
@@ -733,27 +712,25 @@ extern "C" int vista_run(vista_stack *h)
         a.count = h->count;
         a.stats = h->stats;
         a.err = h->err;
-        if (!fp64) {
-            SortArgs &so = a.so;
-            const SortLayout &L = layouts[ci];
-            char *b = (char *)h->b_sort.p;
-            so.hist = (uint32_t *)(b + L.hist);
-            so.qstart = (uint32_t *)(b + L.qstart);
-            so.ioff = (int64_t *)(b + L.ioff);
-            so.segcnt = (uint32_t *)(b + L.segcnt);
-            so.slot = (uint32_t *)(b + L.slot);
-            so.key = (uint32_t *)(b + L.key);
-            so.perm = (uint32_t *)(b + L.perm);
-            so.tmp = (unsigned long long *)(b + L.tmp);
-            so.items = (Item *)(b + L.items);
-            so.ctr = (uint32_t *)(b + L.ctr);
-            so.sorted = cfg.sort_rows;
-            so.stripe_rows = cfg.sort_rows ? h->stripe_rows : c.nv;
-            so.nstripe = cfg.sort_rows ? h->nstripe : 1;
-            so.ushift = h->ushift;
-            so.nuk = h->nuk;
-            so.rows_per_item = cfg.rows_per_item;
-        }
+        SortArgs &so = a.so;
+        const SortLayout &L = layouts[ci];
+        char *b = (char *)h->b_sort.p;
+        so.hist = (uint32_t *)(b + L.hist);
+        so.qstart = (uint32_t *)(b + L.qstart);
+        so.ioff = (int64_t *)(b + L.ioff);
+        so.segcnt = (uint32_t *)(b + L.segcnt);
+        so.slot = (uint32_t *)(b + L.slot);
+        so.key = (uint32_t *)(b + L.key);
+        so.perm = (uint32_t *)(b + L.perm);
+        so.tmp = (unsigned long long *)(b + L.tmp);
+        so.items = (Item *)(b + L.items);
+        so.ctr = (uint32_t *)(b + L.ctr);
+        so.sorted = cfg.sort_rows;
+        so.stripe_rows = cfg.sort_rows ? h->stripe_rows : c.nv;
+        so.nstripe = cfg.sort_rows ? h->nstripe : 1;
+        so.ushift = h->ushift;
+        so.nuk = h->nuk;
+        so.rows_per_item = cfg.rows_per_item;
     }
     h->classes = std::move(classes);
     h->copies = std::move(copies);
