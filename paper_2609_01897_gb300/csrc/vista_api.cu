@@ -32,7 +32,7 @@ int stripe_geometry(vista_stack *h)
 {
     const vista_cube_desc &d = h->desc;
     int S = 1, nst = 1, ushift = 0, nuk = 1;
-    if (!stripe_layout(d.nu, d.nv, d.nrest, d.npol, &S, &nst, &ushift, &nuk)) return VISTA_E_RANGE;
+    if (!stripe_layout(d.nu, d.nv, d.nrest, d.npol, MIN_STRIPES, &S, &nst, &ushift, &nuk)) return VISTA_E_RANGE;
     h->stripe_rows = S;
     h->nstripe = nst;
     h->ushift = ushift;

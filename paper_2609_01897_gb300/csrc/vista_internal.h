@@ -11,19 +11,35 @@ namespace vista {
 constexpr double C_LIGHT = 299792458.0;   // m/s
 constexpr int MAX_LOCAL_KEYS = 4096;      // cell keys inside one stripe (shared-memory histogram)
 constexpr int MAX_STRIPES = 4096;         // stripes of the cube (shared-memory running counts)
-constexpr int SEG_ROWS = 2048;            // rows per segment of the row-order slot assignment
+// Rows per segment of the row-order slot assignment: a block's work in three
+// pre-pass kernels.  512 rather than 2048 spreads windows of ten thousand rows
+// over enough blocks (k_keys of twelve ragged windows in three classes 47 ->
+// 21 us, of four windows of 18 000 rows 9.3 -> 4.9 us; level for large ones);
+// the fixed scratch of the no-allocation call holds the counts of 2048-row
+// segments.
+constexpr int SEG_ROWS = 512, SEG_ROWS_NOALLOC = 2048;
+// Stripes a handle's cube is cut into at the least (where it has the rows): a
+// block sorts one (window, stripe) bucket, so that a small cube, whose
+// entries would all fit one stripe, still spreads a window's sort over many
+// blocks (k_bucket_sort of one window of 10 001 rows 31 -> 7 us, of four of
+// 18 000 rows 68 -> 10 us; more, smaller items also fill the chip better when
+// a stack is small).
+constexpr int MIN_STRIPES = 32;
 
 // Row-ordering stripes of a cube: S iv rows per stripe (sized so that a
-// stripe's cube entries, ~20 B each, stay near 40 MB and resident in L2),
-// at most MAX_STRIPES stripes, and a local cell key (iv % S) * nuk + (iu >>
-// ushift) below MAX_LOCAL_KEYS.  Returns false if no such layout exists.
-inline bool stripe_layout(int nu, int nv, int nrest, int npol, int *S_out, int *nst_out, int *ushift_out,
-                          int *nuk_out)
+// stripe's cube entries, ~20 B each, stay near 40 MB and resident in L2, and
+// that there are min_stripes of them), at most MAX_STRIPES stripes, and a
+// local cell key (iv % S) * nuk + (iu >> ushift) below MAX_LOCAL_KEYS.
+// Returns false if no such layout exists.
+inline bool stripe_layout(int nu, int nv, int nrest, int npol, int min_stripes, int *S_out, int *nst_out,
+                          int *ushift_out, int *nuk_out)
 {
     const double row_bytes = (double)nu * nrest * npol * 20.0;
     const int minS = (nv + MAX_STRIPES - 1) / MAX_STRIPES;
     if (minS > MAX_LOCAL_KEYS) return false;
     double s0 = 40e6 / row_bytes;
+    const double most = (double)nv / min_stripes;
+    s0 = s0 > most ? most : s0;
     s0 = s0 < 1.0 ? 1.0 : (s0 > nv ? nv : s0);
     int S = (int)s0 < minS ? minS : (int)s0;
     int ushift = 0, nuk = nu;
@@ -179,7 +195,7 @@ struct LaunchCfg {
 //   tmp      [rows]             (local key << 32) | row, bucket-grouped
 //   perm     [rows]             row of each processing position
 //   ioff     [nbuckets + 1]     first work item of each bucket (stripe-major)
-//   segcnt   [nseg][nstripe]    rows of each (segment of SEG_ROWS rows, stripe), then
+//   segcnt   [nseg][nstripe]    rows of each (segment of seg_rows rows, stripe), then
 //                               the segment's first slot in each bucket
 //   seg_off  [nwin + 1]         cumulative segments per window
 //   items    [max_items]        work list, stripe-major
@@ -199,6 +215,7 @@ struct SortArgs {
     int32_t ushift, nuk;        // local key = (iv % stripe_rows) * nuk + (iu >> ushift)
     int32_t sorted;             // 0: identity order
     int32_t rows_per_item;
+    int32_t seg_rows;           // rows per segment
 };
 
 // Everything one launch class needs on the device.

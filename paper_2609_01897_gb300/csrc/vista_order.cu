@@ -27,7 +27,7 @@
 namespace vista {
 
 // Row-order slots in (window, stripe) buckets, three passes over segments of
-// SEG_ROWS rows: keys and per-segment stripe counts, an exclusive scan of the
+// seg_rows rows: keys and per-segment stripe counts, an exclusive scan of the
 // counts over each window's segments, then each segment's slots in row order
 // (ranks within a warp from a match, warps in turn against running counts in
 // shared memory).  Rows that share a bucket thus keep their row order.
@@ -42,9 +42,9 @@ __device__ __forceinline__ SegRange seg_range(const RunArgs &a, int64_t seg)
     SegRange sr;
     sr.w = find_owner(a.so.seg_off, a.nsrc, seg);
     sr.g0 = a.row_off[sr.w];
-    sr.r0 = (seg - a.so.seg_off[sr.w]) * SEG_ROWS;
+    sr.r0 = (seg - a.so.seg_off[sr.w]) * a.so.seg_rows;
     const int64_t n = a.srcs[sr.w].nrow;
-    sr.r1 = sr.r0 + SEG_ROWS < n ? sr.r0 + SEG_ROWS : n;
+    sr.r1 = sr.r0 + a.so.seg_rows < n ? sr.r0 + a.so.seg_rows : n;
     return sr;
 }
 

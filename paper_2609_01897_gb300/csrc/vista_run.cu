@@ -731,6 +731,7 @@ extern "C" int vista_run(vista_stack *h)
         so.ushift = h->ushift;
         so.nuk = h->nuk;
         so.rows_per_item = cfg.rows_per_item;
+        so.seg_rows = SEG_ROWS;
     }
     h->classes = std::move(classes);
     h->copies = std::move(copies);
