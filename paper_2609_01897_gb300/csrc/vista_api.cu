@@ -75,6 +75,15 @@ int cuda_fail(vista_stack *h, cudaError_t e, const char *what)
                 cudaGetErrorString(e));
 }
 
+int finish_with_error_word(vista_stack *h, const char *what)
+{
+    int32_t err = 0;
+    cudaError_t e = cudaMemcpyAsync(&err, h->err, sizeof err, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, what);
+    return err != 0 ? device_fail(h, err) : VISTA_OK;
+}
+
 int device_fail(vista_stack *h, int32_t code)
 {
     if (code == 1) return fail(h, VISTA_E_TIMEOUT, "a device-side wait gave up (code 1)");
@@ -374,12 +383,6 @@ int read_common(vista_stack *h, void *sum_wv, void *sum_w, void *sum_wvv, uint32
 {
     cudaError_t e = finish_readback(h);
     if (e != cudaSuccess) return cuda_fail(h, e, "earlier readback");
-    e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return cuda_fail(h, e, "stream synchronize");
-    int32_t err = 0;
-    e = cudaMemcpy(&err, h->err, sizeof err, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(h, e, "error word read");
-    if (err != 0) return device_fail(h, err);
     const int fp64 = h->desc.precision == VISTA_PREC_FP64;
     const int all = cube_counts_exact(h) ? 0 : 1;
     const int64_t n = h->nentries;
@@ -387,9 +390,8 @@ int read_common(vista_stack *h, void *sum_wv, void *sum_w, void *sum_wvv, uint32
     if (dst_dev) {
         e = launch_unpack(h->cube, h->cube_master, h->count, fp64, all, n, sum_wv, sum_w, sum_wvv, count, out_f64,
                           h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "cube unpack");
-        return VISTA_OK;
+        return finish_with_error_word(h, "cube unpack");
     }
     // host destination: unpack into a device scratch area, then copy
     const size_t b_wv = sum_wv ? (size_t)n * 2 * fe : 0, b_w = sum_w ? (size_t)n * fe : 0,
@@ -409,9 +411,8 @@ int read_common(vista_stack *h, void *sum_wv, void *sum_w, void *sum_wvv, uint32
     if (e == cudaSuccess && sum_wvv) e = cudaMemcpyAsync(sum_wvv, d_vv, b_vv, cudaMemcpyDeviceToHost, h->xfer[2]);
     if (e == cudaSuccess && count) e = cudaMemcpyAsync(count, d_c, b_c, cudaMemcpyDeviceToHost, h->xfer[3]);
     if (e == cudaSuccess) e = xfer_join(h);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "cube readback");
-    return VISTA_OK;
+    return finish_with_error_word(h, "cube readback");
 }
 
 }  // namespace
@@ -496,12 +497,6 @@ extern "C" int vista_read_cube_sparse(vista_stack *h, int64_t cap, int64_t *inde
     if (cap > 0 && !index) return fail(h, VISTA_E_ARG, "null index with cap > 0");
     cudaError_t e = finish_readback(h);
     if (e != cudaSuccess) return cuda_fail(h, e, "earlier readback");
-    e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return cuda_fail(h, e, "stream synchronize");
-    int32_t err = 0;
-    e = cudaMemcpy(&err, h->err, sizeof err, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(h, e, "error word read");
-    if (err != 0) return device_fail(h, err);
     const int fp64 = h->desc.precision == VISTA_PREC_FP64;
     const int64_t n = h->nentries, ntile = sparse_tiles(n);
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
@@ -514,8 +509,8 @@ extern "C" int vista_read_cube_sparse(vista_stack *h, int64_t cap, int64_t *inde
     int64_t total = 0;
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(&total, b + o_tot, sizeof total, cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "sparse readback count");
+    if (const int rc = finish_with_error_word(h, "sparse readback count")) return rc;
     *n_touched = total;
     if (cap == 0) return VISTA_OK;   // the count only
     if (total > cap)
@@ -584,14 +579,14 @@ extern "C" int vista_zero_cube(vista_stack *h)
     const bool fp64 = h->desc.precision == VISTA_PREC_FP64;
     cudaError_t e;
     if (cube_counts_exact(h)) {
-        e = launch_zero_touched(h->cube, h->cube_master, h->count, fp64, h->nentries, h->stream);
+        e = launch_zero_touched(h->cube, h->cube_master, h->count, h->stats, fp64, h->nentries, h->stream);
     } else {
         e = cudaMemsetAsync(h->cube, 0, (size_t)h->nentries * (fp64 ? 32 : 16), h->stream);
         if (e == cudaSuccess && h->cube_master)
             e = cudaMemsetAsync(h->cube_master, 0, (size_t)h->nentries * 32, h->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(h->count, 0, (size_t)h->nentries * 4, h->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(h->stats, 0, sizeof(DevStats), h->stream);
     }
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->stats, 0, sizeof(DevStats), h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "cube zeroing");
     h->host_nvis = 0;
     h->nvis_since_fold = 0;

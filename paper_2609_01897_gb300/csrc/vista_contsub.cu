@@ -541,14 +541,8 @@ extern "C" int vista_contsub(vista_stack *h, const uint8_t *line_free, int32_t o
     const int nrest = h->desc.nrest;
     const size_t n_out = (size_t)h->nentries * sizeof(float2);
     const size_t lf_bytes = ((size_t)nrest + 255) & ~(size_t)255;
-    cudaError_t e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return cuda_fail(h, e, "stream synchronize");
-    int32_t err = 0;
-    e = cudaMemcpy(&err, h->err, sizeof err, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(h, e, "error word read");
-    if (err != 0) return device_fail(h, err);
     // the mask (and, for a host destination, the output) in a handle buffer
-    e = h->b_contsub.ensure(lf_bytes + (dst_is_device ? 0 : n_out));
+    cudaError_t e = h->b_contsub.ensure(lf_bytes + (dst_is_device ? 0 : n_out));
     if (e != cudaSuccess) return cuda_fail(h, e, "continuum subtraction buffer");
     uint8_t *d_lf = (uint8_t *)h->b_contsub.p;
     float2 *d_out = dst_is_device ? reinterpret_cast<float2 *>(sum_wv_out)
@@ -557,7 +551,6 @@ extern "C" int vista_contsub(vista_stack *h, const uint8_t *line_free, int32_t o
     if (e == cudaSuccess) e = launch_contsub(h, d_lf, order, d_out, h->stream);
     if (e == cudaSuccess && !dst_is_device)
         e = cudaMemcpyAsync(sum_wv_out, d_out, n_out, cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "continuum subtraction");
-    return VISTA_OK;
+    return finish_with_error_word(h, "continuum subtraction");
 }

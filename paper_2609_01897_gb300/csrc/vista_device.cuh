@@ -24,6 +24,41 @@ __device__ __forceinline__ int find_owner(const int64_t *__restrict__ off, int n
     return lo;
 }
 
+// ---- programmatic dependent launch ----
+//
+// The pre-pass is a chain of short kernels; each is launched while the one
+// before it still runs (launch_chained) and first waits for that one to end,
+// its writes visible.  Only then does it let its own successor be launched,
+// so that at most two kernels of the chain are on the chip and everything
+// older, the caller's inputs among it, is complete.  About a microsecond a
+// kernel: a test-sized stack's call 160 -> 141 us together with the readback's
+// single wait.  The stacking kernels are launched as usual: their persistent
+// blocks, waiting on the chip before the pre-pass has ended, cost the FP64
+// form 6 % and an archive stack 1 %.
+
+__device__ __forceinline__ void chain_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... KA, typename... A>
+static cudaError_t launch_chained(void (*kern)(KA...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                                  A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // ---- TMA bulk copies into shared memory, completed on an mbarrier ----
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }

@@ -148,6 +148,8 @@ int cuda_fail(vista_stack *h, cudaError_t e, const char *what);
 // A nonzero device error word as a status: 1 a bounded wait gave up
 // (E_TIMEOUT), other codes an internal sizing check (E_STATE).
 int device_fail(vista_stack *h, int32_t code);
+// Waits for the stream, and reports a nonzero error word of the work on it.
+int finish_with_error_word(vista_stack *h, const char *what);
 int span_begin(vista_stack *h, int kind);
 void span_end(vista_stack *h, int id);
 size_t vis_elem_bytes(int vt);

@@ -11,13 +11,15 @@ namespace vista {
 constexpr double C_LIGHT = 299792458.0;   // m/s
 constexpr int MAX_LOCAL_KEYS = 4096;      // cell keys inside one stripe (shared-memory histogram)
 constexpr int MAX_STRIPES = 4096;         // stripes of the cube (shared-memory running counts)
-// Rows per segment of the row-order slot assignment: a block's work in three
-// pre-pass kernels.  512 rather than 2048 spreads windows of ten thousand rows
-// over enough blocks (k_keys of twelve ragged windows in three classes 47 ->
-// 21 us, of four windows of 18 000 rows 9.3 -> 4.9 us; level for large ones);
-// the fixed scratch of the no-allocation call holds the counts of 2048-row
-// segments.
-constexpr int SEG_ROWS = 512, SEG_ROWS_NOALLOC = 2048;
+// Rows per segment of the row-order slot assignment (a block's work in three
+// pre-pass kernels).  2048, or 512 when those would be fewer than two a SM,
+// which spreads windows of ten thousand rows over enough blocks (k_keys of
+// twelve ragged windows in three classes 47 -> 21 us, of four windows of
+// 18 000 rows 9.3 -> 4.9 us; for 23 windows of 108 360 rows the three kernels
+// would take 61 us instead of 48).  The fixed scratch of the no-allocation
+// call holds the counts of 2048-row segments.
+constexpr int SEG_ROWS = 2048, SEG_ROWS_SMALL = 512;
+inline int segment_rows(int64_t rows) { return rows / SEG_ROWS < 2 * 152 ? SEG_ROWS_SMALL : SEG_ROWS; }
 // Stripes a handle's cube is cut into at the least (where it has the rows): a
 // block sorts one (window, stripe) bucket, so that a small cube, whose
 // entries would all fit one stripe, still spreads a window's sort over many
@@ -255,8 +257,9 @@ cudaError_t launch_fold(void *cube, double *master, int64_t n, cudaStream_t st);
 cudaError_t launch_unpack(const void *cube, const double *master, const uint32_t *count, int fp64, int all, int64_t n,
                           void *sum_wv, void *sum_w, void *sum_wvv, uint32_t *cnt_out,
                           int out_f64, cudaStream_t st);
-// Zero the entries whose count is not 0 (all others must be zero).
-cudaError_t launch_zero_touched(void *cube, double *master, uint32_t *count, int fp64, int64_t n, cudaStream_t st);
+// Zero the entries whose count is not 0 (all others must be zero) and the counters.
+cudaError_t launch_zero_touched(void *cube, double *master, uint32_t *count, DevStats *stats, int fp64, int64_t n,
+                                cudaStream_t st);
 // Sparse readback (the entries with count > 0, in entry order): per tile of
 // 4096 entries the touched count (tile_cnt [ntile]), their exclusive scan
 // (tile_off [ntile]) and the total (one int64 on the device); then each

@@ -192,13 +192,14 @@ __global__ void __launch_bounds__(CUBE_THREADS) unpack_kernel(const void *cube, 
 }
 
 // Zeroes the entries whose count is not 0 (every other entry is zero
-// already): the counts are read, 52 bytes of a touched entry are written
-// (mixed).  Against setting the whole cube to zero at the HBM peak: 6.7e7
+// already), and the counters: the counts are read, 52 bytes of a touched
+// entry are written (mixed).  Against setting the whole cube to zero at the HBM peak: 6.7e7
 // entries, 31 % touched, 518 -> 221 us; 2.7e8 entries, 2.6 % touched, 2053 ->
 // 245 us.  A cube touched throughout would cost 4 bytes in 52 more.
-__global__ void __launch_bounds__(CUBE_THREADS) zero_kernel(void *cube, double *master, uint32_t *count, int fp64,
-                                                            int64_t n)
+__global__ void __launch_bounds__(CUBE_THREADS) zero_kernel(void *cube, double *master, uint32_t *count,
+                                                            DevStats *stats, int fp64, int64_t n)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *stats = DevStats{};
     for (int64_t b = (int64_t)blockIdx.x * CUBE_TILE + threadIdx.x; b < n; b += (int64_t)gridDim.x * CUBE_TILE) {
         uint32_t c[CUBE_UNROLL];
 #pragma unroll
@@ -376,10 +377,11 @@ cudaError_t launch_unpack(const void *cube, const double *master, const uint32_t
     return cudaGetLastError();
 }
 
-cudaError_t launch_zero_touched(void *cube, double *master, uint32_t *count, int fp64, int64_t n, cudaStream_t st)
+cudaError_t launch_zero_touched(void *cube, double *master, uint32_t *count, DevStats *stats, int fp64, int64_t n,
+                                cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    zero_kernel<<<cube_blocks(n), CUBE_THREADS, 0, st>>>(cube, master, count, fp64, n);
+    zero_kernel<<<cube_blocks(n), CUBE_THREADS, 0, st>>>(cube, master, count, stats, fp64, n);
     return cudaGetLastError();
 }
 

@@ -186,7 +186,7 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     const size_t o_ioff = o;
     o += al256(8 * ((size_t)nstripe + 1));
     const size_t o_segcnt = o;
-    o += al256(4 * (size_t)((nrow + SEG_ROWS_NOALLOC - 1) / SEG_ROWS_NOALLOC) * (size_t)nstripe);
+    o += al256(4 * (size_t)((nrow + SEG_ROWS - 1) / SEG_ROWS) * (size_t)nstripe);
     const size_t o_slot = o;
     o += al256(4 * (size_t)nrow);
     const size_t o_key = o;
@@ -246,7 +246,7 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     d.key_sv = (float)(s->freqs[key_ch] * gv);
     d.rec_off = 0;
     d.cell_off = 0;
-    const int64_t nseg = (nrow + SEG_ROWS_NOALLOC - 1) / SEG_ROWS_NOALLOC;
+    const int64_t nseg = (nrow + SEG_ROWS - 1) / SEG_ROWS;
     // rows, row segments
     const int64_t roff[4] = {0, nrow, 0, nseg};
 
@@ -298,7 +298,7 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     a.so.nuk = nuk;
     a.so.sorted = 1;
     a.so.rows_per_item = R;
-    a.so.seg_rows = SEG_ROWS_NOALLOC;
+    a.so.seg_rows = SEG_ROWS;
     e = launch_prepare(a, st);
     // one channel per lane, four warps per block, two rows of visibilities in flight
     if (e == cudaSuccess) e = launch_mixed(a, (s->vis_type << 16) | (1 << 8) | s->npol, 4, 2, st);

@@ -52,6 +52,7 @@ __device__ __forceinline__ SegRange seg_range(const RunArgs &a, int64_t seg)
 // (stripe, local cell key), and the stripe counts of the segment.
 __global__ void __launch_bounds__(256) k_keys(RunArgs a)
 {
+    chain_begin();
     __shared__ uint32_t cnt[MAX_STRIPES];
     const SortArgs &so = a.so;
     const int64_t seg = blockIdx.x;
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(256) k_keys(RunArgs a)
 // and the bucket's row count.
 __global__ void __launch_bounds__(256) k_segscan(RunArgs a)
 {
+    chain_begin();
     const SortArgs &so = a.so;
     const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -137,6 +139,7 @@ __global__ void __launch_bounds__(256) k_segscan(RunArgs a)
 // Dynamic shared memory: W x nstripe words.
 __global__ void __launch_bounds__(256) k_slots(RunArgs a)
 {
+    chain_begin();
     extern __shared__ uint32_t dsm[];
     const SortArgs &so = a.so;
     if (!so.sorted) return;
@@ -199,13 +202,24 @@ static cudaError_t allow_smem(K kern, size_t smem)
 // One block of 1024 threads.
 __global__ void __launch_bounds__(1024) k_scan(RunArgs a)
 {
+    chain_begin();
     const SortArgs &so = a.so;
     const int nw = a.nsrc, ns = so.nstripe, R = so.rows_per_item;
-    for (int w = threadIdx.x; w < nw; w += blockDim.x) {
-        uint32_t acc = 0;
-        for (int s = 0; s < ns; ++s) {
-            so.qstart[(size_t)w * ns + s] = acc;
-            acc += so.hist[(size_t)w * ns + s];
+    // a warp per window: its buckets' first positions, 32 stripes at a time
+    const int lane = threadIdx.x & 31;
+    for (int w = threadIdx.x >> 5; w < nw; w += blockDim.x >> 5) {
+        uint32_t run = 0;
+        for (int s0 = 0; s0 < ns; s0 += 32) {
+            const int s = s0 + lane;
+            const uint32_t n = s < ns ? so.hist[(size_t)w * ns + s] : 0u;
+            uint32_t incl = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (s < ns) so.qstart[(size_t)w * ns + s] = run + incl - n;
+            run += __shfl_sync(0xffffffffu, incl, 31);
         }
     }
     __syncthreads();
@@ -213,11 +227,15 @@ __global__ void __launch_bounds__(1024) k_scan(RunArgs a)
     const int64_t nb = (int64_t)nw * ns;
     const int64_t per = (nb + blockDim.x - 1) / blockDim.x;
     const int64_t i0 = min(nb, (int64_t)threadIdx.x * per), i1 = min(nb, i0 + per);
+    const int s_first = (int)(i0 / nw), w_first = (int)(i0 % nw);
     int64_t local = 0;
-    for (int64_t i = i0; i < i1; ++i) {
-        const int s = (int)(i / nw), w = (int)(i % nw);
-        const int64_t n = so.hist[(size_t)w * ns + s];
-        local += ((n + R - 1) / R) * a.srcs[w].nchunk;
+    for (int64_t i = i0, s = s_first, w = w_first; i < i1; ++i) {
+        const uint32_t n = so.hist[(size_t)w * ns + s];
+        local += (int64_t)((n + R - 1) / R) * a.srcs[w].nchunk;
+        if (++w == nw) {
+            w = 0;
+            ++s;
+        }
     }
     __shared__ long long part[1024];
     part[threadIdx.x] = local;
@@ -230,11 +248,14 @@ __global__ void __launch_bounds__(1024) k_scan(RunArgs a)
     }
     int64_t pos = part[threadIdx.x] - local;
     const int64_t total = part[blockDim.x - 1];
-    for (int64_t i = i0; i < i1; ++i) {
+    for (int64_t i = i0, s = s_first, w = w_first; i < i1; ++i) {
         so.ioff[i] = pos;
-        const int s = (int)(i / nw), w = (int)(i % nw);
-        const int64_t n = so.hist[(size_t)w * ns + s];
-        pos += ((n + R - 1) / R) * a.srcs[w].nchunk;
+        const uint32_t n = so.hist[(size_t)w * ns + s];
+        pos += (int64_t)((n + R - 1) / R) * a.srcs[w].nchunk;
+        if (++w == nw) {
+            w = 0;
+            ++s;
+        }
     }
     if (threadIdx.x == 0) so.ioff[nb] = total;
     if (threadIdx.x == 0) {
@@ -249,6 +270,7 @@ __global__ void __launch_bounds__(1024) k_scan(RunArgs a)
 // into the window's channel chunks.
 __global__ void __launch_bounds__(256) k_items(RunArgs a)
 {
+    chain_begin();
     const SortArgs &so = a.so;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nb = (int64_t)a.nsrc * so.nstripe;
@@ -278,6 +300,7 @@ __global__ void __launch_bounds__(256) k_items(RunArgs a)
 
 __global__ void __launch_bounds__(256) k_scatter(RunArgs a)
 {
+    chain_begin();
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= a.nrows_total) return;
     const SortArgs &so = a.so;
@@ -300,6 +323,7 @@ __global__ void __launch_bounds__(256) k_scatter(RunArgs a)
 // Dynamic shared memory: (W + 1) x nk words.
 __global__ void __launch_bounds__(256) k_bucket_sort(RunArgs a)
 {
+    chain_begin();
     extern __shared__ uint32_t dsm[];
     __shared__ uint32_t part[256];
     const SortArgs &so = a.so;
@@ -485,6 +509,7 @@ __device__ int2 chunk_cell(const RunArgs &a, const SrcDev &S, const ChanF *cf, c
 // is formed: one load latency per chunk overlaps the previous chunk's work.
 __global__ void __launch_bounds__(256) k_rows(RunArgs a)
 {
+    chain_begin();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.nrows_total) return;
     const int w = find_owner(a.row_off, a.nsrc, p);
@@ -524,46 +549,35 @@ __global__ void __launch_bounds__(256) k_rows(RunArgs a)
 cudaError_t launch_prepare(const RunArgs &a, cudaStream_t st, int *nlaunch)
 {
     const SortArgs &so = a.so;
-    int n = 0;
-    cudaError_t e = cudaMemsetAsync(so.hist, 0, sizeof(uint32_t) * (size_t)a.nsrc * so.nstripe, st);
-    if (e != cudaSuccess) return e;
+    if (nlaunch) *nlaunch = 0;
+    if (so.nseg_total == 0 || a.nrows_total == 0) return cudaErrorInvalidValue;   // (a class has rows)
     const unsigned rb = (unsigned)((a.nrows_total + 255) / 256);
-    if (so.nseg_total > 0) {
-        k_keys<<<(unsigned)so.nseg_total, 256, 0, st>>>(a);
-        const int64_t nb = (int64_t)a.nsrc * so.nstripe;
-        k_segscan<<<(unsigned)((nb * 32 + 255) / 256), 256, 0, st>>>(a);
-        const int nws = table_warps(so.nstripe, 0);
-        const size_t smem_s = (size_t)nws * so.nstripe * sizeof(uint32_t);
-        const cudaError_t ea = allow_smem(k_slots, smem_s);
-        if (ea != cudaSuccess) return ea;
-        k_slots<<<(unsigned)so.nseg_total, 32 * nws, smem_s, st>>>(a);
-        n += 3;
-    }
-    k_scan<<<1, 1024, 0, st>>>(a);
+    const int64_t nb = (int64_t)a.nsrc * so.nstripe;
+    const int nws = table_warps(so.nstripe, 0);
+    const size_t smem_s = (size_t)nws * so.nstripe * sizeof(uint32_t);
+    const int nk = so.stripe_rows * so.nuk, nwb = table_warps(nk, 1);
+    const size_t smem_b = (size_t)(nwb + 1) * nk * sizeof(uint32_t);
+    cudaError_t e = allow_smem(k_slots, smem_s);
+    if (e == cudaSuccess) e = allow_smem(k_bucket_sort, smem_b);
+    if (e != cudaSuccess) return e;
+    int n = 0;
+    k_keys<<<(unsigned)so.nseg_total, 256, 0, st>>>(a);
+    e = cudaGetLastError();
+    auto next = [&](void (*kern)(RunArgs), int64_t grid, unsigned block, size_t smem) {
+        if (e != cudaSuccess) return;
+        e = launch_chained(kern, (unsigned)grid, block, smem, st, a);
+        ++n;
+    };
     ++n;
-    if (so.max_items > 0) {
-        k_items<<<(unsigned)((so.max_items + 255) / 256), 256, 0, st>>>(a);
-        ++n;
-    }
-    if (rb) {
-        k_scatter<<<rb, 256, 0, st>>>(a);
-        ++n;
-    }
-    const int64_t nbuckets = (int64_t)a.nsrc * so.nstripe;
-    if (rb && nbuckets) {
-        const int nk = so.stripe_rows * so.nuk, nw = table_warps(nk, 1);
-        const size_t smem = (size_t)(nw + 1) * nk * sizeof(uint32_t);
-        const cudaError_t ea = allow_smem(k_bucket_sort, smem);
-        if (ea != cudaSuccess) return ea;
-        k_bucket_sort<<<(unsigned)nbuckets, 32 * nw, smem, st>>>(a);
-        ++n;
-    }
-    if (rb) {
-        k_rows<<<rb, 256, 0, st>>>(a);
-        ++n;
-    }
+    next(k_segscan, (nb * 32 + 255) / 256, 256, 0);
+    next(k_slots, so.nseg_total, 32 * (unsigned)nws, smem_s);
+    next(k_scan, 1, 1024, 0);
+    next(k_items, (so.max_items + 255) / 256, 256, 0);
+    next(k_scatter, rb, 256, 0);
+    next(k_bucket_sort, nb, 32 * (unsigned)nwb, smem_b);
+    next(k_rows, rb, 256, 0);
     if (nlaunch) *nlaunch = n;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace vista

@@ -554,7 +554,10 @@ extern "C" int vista_run(vista_stack *h)
         cls_off0[ci] = offs.size();
         const size_t m = cr.members.size();
         std::vector<int64_t> roff(m + 1, 0), soff(m + 1, 0);
-        int64_t max_items = 0;
+        int64_t max_items = 0, class_rows = 0;
+        for (int i : cr.members) class_rows += h->pending[(size_t)i].d.nrow;
+        const int seg = segment_rows(class_rows);
+        cr.args.so.seg_rows = seg;
         for (size_t t = 0; t < m; ++t) {
             const int i = cr.members[t];
             const SrcHost &s = h->pending[(size_t)i];
@@ -647,7 +650,7 @@ extern "C" int vista_run(vista_stack *h)
                 bound_run += entry_bound(s, pl);
             }
             roff[t + 1] = roff[t] + d.nrow;
-            soff[t + 1] = soff[t] + (d.nrow + SEG_ROWS - 1) / SEG_ROWS;
+            soff[t + 1] = soff[t] + (d.nrow + seg - 1) / seg;
             max_items += (int64_t)d.nchunk * ((d.nrow + cfg.rows_per_item - 1) / cfg.rows_per_item + h->nstripe);
             d.guvw = d.uvw;
             if (s.has_rot) {
@@ -731,7 +734,6 @@ extern "C" int vista_run(vista_stack *h)
         so.ushift = h->ushift;
         so.nuk = h->nuk;
         so.rows_per_item = cfg.rows_per_item;
-        so.seg_rows = SEG_ROWS;
     }
     h->classes = std::move(classes);
     h->copies = std::move(copies);
