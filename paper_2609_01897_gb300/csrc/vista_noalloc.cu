@@ -110,7 +110,7 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     int rc = channel_bins(s->freqs, n, s->z, c->rest_f0, c->rest_df, c->nrest, c->bin_mode, j0.data(), nb.data(),
                           w.data());
     if (rc != VISTA_OK) return fail(nullptr, rc, "channel planning failed");
-    int32_t lo = -1, hi = -1, key_ch = 0;
+    int32_t lo = -1, hi = -1;
     for (int32_t k = 0; k < n; ++k)
         if (nb[(size_t)k] > 0) {
             if (lo < 0) lo = k;
@@ -127,7 +127,6 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     const int32_t nin = hi - lo;
     std::vector<ChanF> chf((size_t)nin);
     std::vector<ChanD> chd((size_t)nin);
-    double fbest = -1.0;
     for (int32_t k = lo; k < hi; ++k) {
         ChanD &d = chd[(size_t)(k - lo)];
         ChanF &f = chf[(size_t)(k - lo)];
@@ -146,10 +145,6 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
         const double nuc = d.nu / C_LIGHT;
         f.nuc_hi = (float)nuc;
         f.nuc_lo = (float)(nuc - (double)f.nuc_hi);
-        if (std::fabs(d.nu) > fbest) {
-            fbest = std::fabs(d.nu);
-            key_ch = k;
-        }
     }
     double step = 0.0;
     const bool linear = linear_axis(s->freqs, n, &step);
@@ -242,6 +237,7 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     d.nchunk = nchunk;
     d.vstride = n;
     d.kbase = 0;
+    const int32_t key_ch = lo + nin / 2;   // rows are ordered by their cell at the middle channel
     d.key_su = (float)(s->freqs[key_ch] * gu);
     d.key_sv = (float)(s->freqs[key_ch] * gv);
     d.rec_off = 0;

@@ -5,10 +5,13 @@
 // work list walks the cube stripe by stripe (a stripe = a few iv rows of the
 // cube, sized to stay resident in L2) across all windows.
 //
-//   k_keys         cell of every row at the window's highest in-cube
-//                  frequency -> (stripe, local cell key); stripe counts per
-//                  segment of rows; a re-projected window's gridding
-//                  baselines R (u, v, w) (Eq. 1)
+//   k_keys         cell of every row at the window's middle in-cube channel
+//                  (from where a row's cell moves least towards both ends of
+//                  the band: 3 to 11 % fewer finished runs than at the highest
+//                  frequency on narrow bands, 4 % more on a 20 % wide one) ->
+//                  (stripe, local cell key); stripe counts per segment of
+//                  rows; a re-projected window's gridding baselines
+//                  R (u, v, w) (Eq. 1)
 //   k_segscan      segment offsets inside each (window, stripe) bucket (a
 //                  warp scan per bucket)
 //   k_slots        each row's slot in its bucket, in row order
@@ -20,8 +23,10 @@
 //   k_bucket_sort  one block per bucket: stable counting sort by local cell
 //                  key (the rows of one key stay in row order), one
 //                  contiguous part of the bucket per warp
-//   k_rows         per row, in processing order: the FP64 delay of Eq. 2 as
-//                  a float-float pair, the weights, and the uv cells of each of the window's channel chunks
+//   k_rows         per row, in processing order (rows of one cell by the part
+//                  of the cell they lie in, see part_order): the FP64 delay of
+//                  Eq. 2 as a float-float pair, the weights, and the uv cells
+//                  of each of the window's channel chunks
 #include "vista_device.cuh"
 
 namespace vista {
@@ -48,7 +53,7 @@ __device__ __forceinline__ SegRange seg_range(const RunArgs &a, int64_t seg)
     return sr;
 }
 
-// Pass 1: the cell of every row at the window's highest in-cube frequency ->
+// Pass 1: the cell of every row at the window's middle in-cube channel ->
 // (stripe, local cell key), and the stripe counts of the segment.
 __global__ void __launch_bounds__(256) k_keys(RunArgs a)
 {
@@ -499,6 +504,52 @@ __device__ int2 chunk_cell(const RunArgs &a, const SrcDev &S, const ChanF *cf, c
     return make_int2(((int)fv0 + (a.g.nv >> 1)) * a.g.nu + ((int)fu0 + (a.g.nu >> 1)), (int)m);
 }
 
+// Rows of one cell by the part of the cell they lie in.  The cell rows are
+// sorted by is that of one channel; at another channel the cell borders run
+// through that cell, and rows that alternate between its parts end a run each
+// time.  In row order they alternate or not as the data have it (the tracks
+// of baselines that share a cell cross a border together when they are sampled
+// densely, and then row order is the better one), so the lanes of a warp, 32
+// rows in processing order, decide on what they see: with T changes of part
+// from row to row inside the cells and G the fewest the parts present allow,
+// the rows of each cell are put in the order of the parts if T > 2 G.  Parts
+// are columns of a third of a cell, walked up and down in turn in two halves
+// (so that neighbouring parts, also of the next cell, follow each other).
+// Finished runs, with the key at the middle channel: compact array 4.49 -> 4.30
+// per 32 rows x channels, wideband 5.49 -> 2.96, long baselines 3.58 -> 3.55,
+// archive 2.34 -> 2.28, ragged 3.98 -> 3.56.  Kernel times with this and the
+// middle channel's key, against the highest frequency's: compact array 1.675
+// -> 1.605 ms, wideband 2.24 -> 1.90, long baselines 1.178 -> 1.141, archive
+// 23.7 -> 23.2, ragged 0.157 -> 0.128; k_rows itself is within 2 %.
+//
+// Returns the row's place among the warp's rows (a permutation of the lanes
+// `act`, 0 ... n - 1; only rows of one window and one cell change places).
+__device__ __forceinline__ int part_order(unsigned act, int w, float x, float y)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const float cx = floorf(x), cy = floorf(y);
+    const int col = min(max((int)((x - cx) * 3.0f), 0), 2), half = y - cy >= 0.5f ? 1 : 0;   // (NaN: 0)
+    const int part = 2 * col + (half ^ (((int)cx + col) & 1));
+    const int pw = __shfl_up_sync(act, w, 1), pp = __shfl_up_sync(act, part, 1);
+    const float px = __shfl_up_sync(act, cx, 1), py = __shfl_up_sync(act, cy, 1);
+    const bool head = lane == 0 || pw != w || px != cx || py != cy;
+    const unsigned heads = __ballot_sync(act, head);
+    const int T = __popc(__ballot_sync(act, !head && pp != part));
+    if (T < 3) return lane;   // (G >= 1 if T >= 1)
+    const int first = 31 - __clz(heads & (below | 1u << lane));
+    const unsigned later = heads & ~(below | 1u << lane);
+    unsigned same = act & ~((1u << first) - 1u) & (later ? (later & (0u - later)) - 1u : 0xffffffffu), less = 0u;
+#pragma unroll
+    for (int b = 4; b > 0; b >>= 1) {
+        const unsigned set = __ballot_sync(act, (part & b) != 0);
+        if (part & b) less |= same & ~set;
+        same &= part & b ? set : ~set;
+    }
+    const int G = __popc(__ballot_sync(act, (same & below) == 0u)) - __popc(heads);
+    return T > 2 * G ? first + __popc(less) + __popc(same & below) : lane;
+}
+
 // One thread per row, in processing order: the row record (the FP64 delay
 // of Eq. 2 as a float-float pair, the weights, the row index)
 // and the chunk-cell entries of all the window's chunks, laid out
@@ -511,16 +562,23 @@ __global__ void __launch_bounds__(256) k_rows(RunArgs a)
 {
     chain_begin();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned act = __ballot_sync(0xffffffffu, p < a.nrows_total);
     if (p >= a.nrows_total) return;
     const int w = find_owner(a.row_off, a.nsrc, p);
     const SrcDev &S = a.srcs[w];
-    const int64_t q = p - a.row_off[w];
     const int64_t r = a.so.perm[p];
     const double *uvw = S.uvw + 3 * r;     // the stored baseline: the delay of Eq. 2
     const double *guvw = S.guvw + 3 * r;   // the gridding baseline (rotated for a re-projected window)
     const double tau = uvw[0] * S.l + uvw[1] * S.m + uvw[2] * S.n1;
     const double u = guvw[0], v = guvw[1];
     const bool fold = a.g.fold && (v < 0.0 || (v == 0.0 && u < 0.0));
+    const float uf = (float)(fold ? -u : u), vf = (float)(fold ? -v : v);
+    int64_t q = p - a.row_off[w];
+    if (a.so.sorted) {
+        const int lane = threadIdx.x & 31, place = part_order(act, w, __fmul_rn(uf, S.key_su), __fmul_rn(vf, S.key_sv));
+        q += place - lane;
+        if (place != lane) a.so.perm[p + place - lane] = (uint32_t)r;   // (every lane has its row)
+    }
     RowRec rec;
     split_ff(fold ? -tau : tau, rec.tau_hi, rec.tau_lo);
     rec.row = (uint32_t)r;
@@ -532,7 +590,6 @@ __global__ void __launch_bounds__(256) k_rows(RunArgs a)
     }
     a.recs[S.rec_off + q] = rec;
 
-    const float uf = (float)(fold ? -u : u), vf = (float)(fold ? -v : v);
     const ChanD *cd = a.chd + S.chan_off;
     const ChanF *cf = a.chf + S.chan_off;
     int2 *out = a.ccells + S.cell_off + q;

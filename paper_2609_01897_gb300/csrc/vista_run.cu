@@ -26,7 +26,7 @@ namespace {
 
 struct Plan {
     int32_t k_lo = 0, k_hi = 0;
-    int32_t key_ch = 0;       // in-cube channel with the largest |frequency|
+    int32_t key_ch = 0;       // the middle in-cube channel: rows are ordered by their cell there
     bool linear = true;
     double step = 0.0;
     int32_t bin_ch = 0;       // the largest number of channels that touch one rest bin
@@ -62,10 +62,10 @@ int plan_source(vista_stack *h, const SrcHost &s, double gu, double gv, Plan &pl
     }
     pl.k_lo = lo;
     pl.k_hi = hi;
+    pl.key_ch = lo + (hi - lo) / 2;
     pl.linear = linear_axis(s.freqs.data(), n, &pl.step);
     pl.chf.resize((size_t)(hi - lo));
     pl.chd.resize((size_t)(hi - lo));
-    double fbest = -1.0;
     for (int32_t k = lo; k < hi; ++k) {
         ChanD &d = pl.chd[(size_t)(k - lo)];
         ChanF &f = pl.chf[(size_t)(k - lo)];
@@ -84,10 +84,6 @@ int plan_source(vista_stack *h, const SrcHost &s, double gu, double gv, Plan &pl
         const double nuc = d.nu / C_LIGHT;   // nu_k / c as a float-float pair
         f.nuc_hi = (float)nuc;
         f.nuc_lo = (float)(nuc - (double)f.nuc_hi);
-        if (std::fabs(d.nu) > fbest) {
-            fbest = std::fabs(d.nu);
-            pl.key_ch = k;
-        }
     }
     // channels per bin, from a difference array over the bins
     std::vector<int32_t> open((size_t)h->desc.nrest + 1, 0);
