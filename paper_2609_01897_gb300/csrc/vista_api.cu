@@ -792,7 +792,7 @@ int debug_common(vista_stack *h, int32_t src, double *ph, int32_t *cells)
     for (const ClassRun &cr : h->classes) {
         for (size_t t = 0; t < cr.members.size(); ++t) {
             if (cr.members[t] != src) continue;
-            cudaError_t e = launch_debug(cr.args, cr.ns, (int)t, h->desc.precision == VISTA_PREC_FP64, ph, cells,
+            cudaError_t e = launch_debug(cr.args, cr.ns, cr.w0 + (int)t, h->desc.precision == VISTA_PREC_FP64, ph, cells,
                                          h->stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "debug export");
@@ -828,7 +828,7 @@ extern "C" int vista_debug_order(vista_stack *h, int32_t src, int32_t *dst)
     for (size_t t = 0; t < cr.members.size(); ++t) {
         if (cr.members[t] != src) continue;
         int64_t off[2];
-        cudaError_t e = cudaMemcpy(off, cr.args.row_off + t, sizeof off, cudaMemcpyDeviceToHost);
+        cudaError_t e = cudaMemcpy(off, cr.args.row_off + cr.w0 + t, sizeof off, cudaMemcpyDeviceToHost);
         if (e == cudaSuccess)
             e = cudaMemcpy(dst, cr.args.so.perm + off[0], sizeof(int32_t) * (size_t)(off[1] - off[0]),
                            cudaMemcpyDeviceToDevice);

@@ -106,12 +106,12 @@ __global__ void __launch_bounds__(32 * WARPS64, 3) stack_fp64_runs(RunArgs a)
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     Warp64<P> &T = reinterpret_cast<Warp64<P> *>(smem)[wid];
-    const uint32_t nitems = a.so.ctr[0], G = gridDim.x * WARPS64;
+    const uint32_t nitems = a.so.ctr[a.cls + 1], G = gridDim.x * WARPS64;   // end of the class's items
     const int npol_c = a.g.npol, nrest = a.g.nrest, gnu = a.g.nu, gnv = a.g.nv;
     double *cube = reinterpret_cast<double *>(a.cube);
     unsigned long long n_read = 0, n_ok = 0, n_duv = 0;
 
-    for (uint32_t it = blockIdx.x * WARPS64 + wid; it < nitems; it += G) {
+    for (uint32_t it = a.so.ctr[a.cls] + blockIdx.x * WARPS64 + wid; it < nitems; it += G) {
         const Item I = a.so.items[it];
         const SrcDev &S = a.srcs[I.w];
         const int n = I.q1 - I.q0, nch = I.nch, kc = min(lane, nch - 1);

@@ -72,6 +72,13 @@ struct ClassRun {
     int wave = 0;                   // host-memory runs: the wave of windows the class belongs to
     RunArgs args{};
     std::vector<int> members;       // run-order index of each window
+    int w0 = 0;                     // first of its windows in the pre-pass
+};
+
+// The pre-pass of the classes [c0, c1) of a run (those of one wave).
+struct PrepRun {
+    RunArgs args{};
+    size_t c0 = 0, c1 = 0;
 };
 
 struct Span {
@@ -101,6 +108,7 @@ struct vista_stack {
     vista::DevBuf b_srcs, b_chf, b_chd, b_recs, b_cells, b_off, b_stage, b_unpack, b_sort, b_rot, b_guvw, b_regrid,
         b_contsub, b_sparse;
     std::vector<vista::ClassRun> classes;
+    std::vector<vista::PrepRun> preps;
     std::vector<vista::Copy2D> copies;   // device copies of the last planned run
     std::vector<vista::HostCopy> hcopies;   // host-memory windows of the last run, by wave
     int nwaves = 0;                      // waves of host-memory windows of the last run (0: none)

@@ -129,7 +129,7 @@ struct SrcDev {
     const uint8_t *fbase;
     int64_t fpitch;
     int32_t fk0;
-    int32_t pad3;
+    int32_t cw;             // channels per chunk (32 * NS of the window's class)
     int64_t pad4;
 };
 static_assert(sizeof(SrcDev) % 16 == 0, "SrcDev is copied in 16-byte units");
@@ -189,24 +189,28 @@ struct LaunchCfg {
     int32_t prefetch_rows;      // visibility rows in flight per warp (2, 4, 8)
 };
 
-// Row ordering of one launch class (device buffers, see vista_kernels.cu).
+// Row ordering of the windows of one pre-pass, in classes (device buffers,
+// see vista_order.cu; bucket i counts class by class, stripe by stripe in a
+// class, window by window in a stripe).
 //   hist     [nwin][nstripe]    rows per (window, stripe)
 //   qstart   [nwin][nstripe]    first processing position of each bucket
 //   slot     [rows]             arrival slot of the row inside its bucket
 //   key      [rows]             stripe << 13 | local cell key
 //   tmp      [rows]             (local key << 32) | row, bucket-grouped
 //   perm     [rows]             row of each processing position
-//   ioff     [nbuckets + 1]     first work item of each bucket (stripe-major)
+//   ioff     [nbuckets + 1]     first work item of each bucket
 //   segcnt   [nseg][nstripe]    rows of each (segment of seg_rows rows, stripe), then
 //                               the segment's first slot in each bucket
 //   seg_off  [nwin + 1]         cumulative segments per window
-//   items    [max_items]        work list, stripe-major
-//   ctr      [2]                item count, queue head
+//   items    [max_items]        work list
+//   ctr      [nclass + 1]       first work item of each class, their number
+//   cls_off  [nclass + 1]       first window of each class
 struct SortArgs {
     uint32_t *hist, *qstart, *slot, *key, *perm;
     int64_t *ioff;
     uint32_t *segcnt;
-    const int64_t *seg_off;
+    const int64_t *seg_off, *cls_off;
+    int32_t nclass;
     int64_t nseg_total;
     unsigned long long *tmp;
     Item *items;
@@ -220,11 +224,13 @@ struct SortArgs {
     int32_t seg_rows;           // rows per segment
 };
 
-// Everything one launch class needs on the device.
+// Everything a pre-pass, and the stacking kernel of each of its classes, needs
+// on the device: cls and cw are the class's.
 struct RunArgs {
     const SrcDev *srcs;
     int32_t nsrc;
-    int32_t cw;                 // channels per chunk (32 * NS) of this class
+    int32_t cls;
+    int32_t cw;                 // channels per chunk (32 * NS)
     const ChanF *chf;
     const ChanD *chd;
     RowRec *recs;
@@ -244,7 +250,7 @@ struct RunArgs {
 };
 
 // Kernel launchers (vista_kernels.cu).  Return a cudaError_t.
-// Row ordering, records and work list of one mixed class (several kernels).
+// Row ordering, records and work list of all classes' windows (several kernels).
 cudaError_t launch_prepare(const RunArgs &a, cudaStream_t st, int *nlaunch = nullptr);   // kernels launched
 // Persistent stacking kernel of one mixed class; key = (vis_type << 16) |
 // (chans_per_lane << 8) | npol, shared by every window of the class.

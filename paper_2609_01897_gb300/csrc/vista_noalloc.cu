@@ -163,7 +163,7 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     const size_t o_src = o;
     o += al256(sizeof(SrcDev));
     const size_t o_off = o;
-    o += al256(4 * sizeof(int64_t));
+    o += al256(6 * sizeof(int64_t));
     const size_t o_chf = o;
     o += al256(sizeof(ChanF) * (size_t)nin);
     const size_t o_chd = o;
@@ -235,6 +235,7 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     d.linear = linear ? 1 : 0;
     for (int p = 0; p < 4; ++p) d.plane[p] = planes[p];
     d.nchunk = nchunk;
+    d.cw = cw;
     d.vstride = n;
     d.kbase = 0;
     const int32_t key_ch = lo + nin / 2;   // rows are ordered by their cell at the middle channel
@@ -243,8 +244,8 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     d.rec_off = 0;
     d.cell_off = 0;
     const int64_t nseg = (nrow + SEG_ROWS - 1) / SEG_ROWS;
-    // rows, row segments
-    const int64_t roff[4] = {0, nrow, 0, nseg};
+    // rows, row segments, the class's windows
+    const int64_t roff[6] = {0, nrow, 0, nseg, 0, 1};
 
     // tables into scratch; counters and the error word start at zero
     e = cudaMemcpyAsync(b + o_src, &d, sizeof d, cudaMemcpyHostToDevice, st);
@@ -268,6 +269,8 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     a.ccells = (int2 *)(b + o_cells);
     a.row_off = (const int64_t *)(b + o_off);
     a.so.seg_off = a.row_off + 2;
+    a.so.cls_off = a.row_off + 4;
+    a.so.nclass = 1;
     a.so.nseg_total = nseg;
     a.nrows_total = nrow;
     a.g = CubeGeom{c->nu, c->nv, c->nrest, c->npol, gu, gv, c->hermitian_fold, 0};

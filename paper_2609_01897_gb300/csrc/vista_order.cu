@@ -16,7 +16,7 @@
 //                  warp scan per bucket)
 //   k_slots        each row's slot in its bucket, in row order
 //   k_scan         one block: per-window bucket offsets, per-bucket work-list
-//                  offsets in stripe-major order (item = rows of one bucket x
+//                  offsets, class by class in stripe-major order (item = rows of one bucket x
 //                  one chunk)
 //   k_items        the work list, one thread per item
 //   k_scatter      rows grouped by bucket
@@ -204,6 +204,21 @@ static cudaError_t allow_smem(K kern, size_t smem)
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
+// The window and stripe of bucket i.
+struct Bucket {
+    int w, s;
+};
+__device__ __forceinline__ Bucket bucket_at(const RunArgs &a, int64_t i)
+{
+    const int ns = a.so.nstripe;
+    if (a.so.nclass == 1) return Bucket{(int)((uint32_t)i % (uint32_t)a.nsrc), (int)((uint32_t)i / (uint32_t)a.nsrc)};
+    int c = 0;
+    while (c + 1 < a.so.nclass && a.so.cls_off[c + 1] * ns <= i) ++c;
+    const int w0 = (int)a.so.cls_off[c], nw = (int)a.so.cls_off[c + 1] - w0;
+    const uint32_t k = (uint32_t)(i - (int64_t)w0 * ns);   // (a class has fewer than 2^31 buckets)
+    return Bucket{w0 + (int)(k % (uint32_t)nw), (int)(k / (uint32_t)nw)};
+}
+
 // One block of 1024 threads.
 __global__ void __launch_bounds__(1024) k_scan(RunArgs a)
 {
@@ -228,51 +243,58 @@ __global__ void __launch_bounds__(1024) k_scan(RunArgs a)
         }
     }
     __syncthreads();
-    // work list in stripe-major order: bucket i = s * nw + w
+    // the work list: four buckets a thread at a time
     const int64_t nb = (int64_t)nw * ns;
-    const int64_t per = (nb + blockDim.x - 1) / blockDim.x;
-    const int64_t i0 = min(nb, (int64_t)threadIdx.x * per), i1 = min(nb, i0 + per);
-    const int s_first = (int)(i0 / nw), w_first = (int)(i0 % nw);
-    int64_t local = 0;
-    for (int64_t i = i0, s = s_first, w = w_first; i < i1; ++i) {
-        const uint32_t n = so.hist[(size_t)w * ns + s];
-        local += (int64_t)((n + R - 1) / R) * a.srcs[w].nchunk;
-        if (++w == nw) {
-            w = 0;
-            ++s;
+    __shared__ long long part[32];
+    long long run = 0;
+    for (int64_t t0 = 0; t0 < nb; t0 += 4 * blockDim.x) {
+        const int64_t i0 = t0 + 4 * threadIdx.x;
+        long long cnt[4], mine = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            cnt[k] = 0;
+            if (i0 + k < nb) {
+                const Bucket b = bucket_at(a, i0 + k);
+                const uint32_t n = so.hist[(size_t)b.w * ns + b.s];
+                cnt[k] = (long long)((n + R - 1) / R) * a.srcs[b.w].nchunk;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mine += cnt[k];
+        long long incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) part[threadIdx.x >> 5] = incl;
+        __syncthreads();
+        long long before = run;
+        for (int v = 0; v < 32; ++v) {
+            const long long x = part[v];
+            if (v < (int)(threadIdx.x >> 5)) before += x;
+            run += x;
+        }
+        __syncthreads();
+        long long pos = before + incl - mine;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i0 + k < nb) so.ioff[i0 + k] = pos;
+            pos += cnt[k];
         }
     }
-    __shared__ long long part[1024];
-    part[threadIdx.x] = local;
-    __syncthreads();
-    for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-        long long v = threadIdx.x >= (unsigned)off ? part[threadIdx.x - off] : 0;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
-    }
-    int64_t pos = part[threadIdx.x] - local;
-    const int64_t total = part[blockDim.x - 1];
-    for (int64_t i = i0, s = s_first, w = w_first; i < i1; ++i) {
-        so.ioff[i] = pos;
-        const uint32_t n = so.hist[(size_t)w * ns + s];
-        pos += (int64_t)((n + R - 1) / R) * a.srcs[w].nchunk;
-        if (++w == nw) {
-            w = 0;
-            ++s;
-        }
-    }
-    if (threadIdx.x == 0) so.ioff[nb] = total;
     if (threadIdx.x == 0) {
-        if (total > so.max_items) atomicExch(a.err, 2);   // host sizing bug: never expected
-        so.ctr[0] = (uint32_t)min(total, so.max_items);
-        so.ctr[1] = 0u;
+        so.ioff[nb] = run;
+        if (run > so.max_items) atomicExch(a.err, 2);   // host sizing bug: never expected
     }
+    __syncthreads();
+    for (int c = threadIdx.x; c <= so.nclass; c += blockDim.x)
+        so.ctr[c] = (uint32_t)min(so.ioff[so.cls_off[c] * ns], so.max_items);
 }
 
-// One thread per work item: bucket i (stripe-major) holds items
-// [ioff[i], ioff[i+1]), rows in groups of rows_per_item, each group split
-// into the window's channel chunks.
+// One thread per work item: bucket i holds items [ioff[i], ioff[i+1]), rows
+// in groups of rows_per_item, each group split into the window's channel
+// chunks.
 __global__ void __launch_bounds__(256) k_items(RunArgs a)
 {
     chain_begin();
@@ -281,22 +303,23 @@ __global__ void __launch_bounds__(256) k_items(RunArgs a)
     const int64_t nb = (int64_t)a.nsrc * so.nstripe;
     if (p >= so.ioff[nb] || p >= so.max_items) return;
     const int i = find_owner(so.ioff, (int)nb, p);
-    const int nw = a.nsrc, R = so.rows_per_item;
-    const int st = i / nw, w = i % nw;
+    const int R = so.rows_per_item;
+    const Bucket bk = bucket_at(a, i);
+    const int st = bk.s, w = bk.w;
     const SrcDev &S = a.srcs[w];
-    const int64_t local = p - so.ioff[i];
-    const int c = (int)(local % S.nchunk);
-    const int64_t t = local / S.nchunk;
+    const uint32_t local = (uint32_t)(p - so.ioff[i]), nchunk = (uint32_t)S.nchunk;   // (a list has fewer than 2^32 items)
+    const uint32_t t = local / nchunk;
+    const int c = (int)(local - t * nchunk);
     const int64_t n = so.hist[(size_t)w * so.nstripe + st];
     const int64_t q = so.qstart[(size_t)w * so.nstripe + st];
     const int nin = S.k_hi - S.k_lo;
     Item it;
     it.w = w;
     it.chunk = c;
-    it.q0 = (int32_t)(q + t * R);
-    it.q1 = (int32_t)min(q + n, q + (t + 1) * R);
-    it.chf0 = S.chan_off + c * a.cw;
-    it.nch = min(a.cw, nin - c * a.cw);
+    it.q0 = (int32_t)(q + (int64_t)t * R);
+    it.q1 = (int32_t)min(q + n, q + ((int64_t)t + 1) * R);
+    it.chf0 = S.chan_off + c * S.cw;
+    it.nch = min(S.cw, nin - c * S.cw);
     it.rec0 = S.rec_off + it.q0;
     it.cell0 = S.cell_off + (int64_t)c * S.nrow + it.q0;
     it.pad = 0;
@@ -420,9 +443,9 @@ __device__ __forceinline__ float2 chan_scales(const ChanF *cf, int k)
 struct ChunkEnds {
     float2 s0, s1;
 };
-__device__ __forceinline__ ChunkEnds chunk_ends(const RunArgs &a, const ChanF *cf, int nin, int c)
+__device__ __forceinline__ ChunkEnds chunk_ends(const ChanF *cf, int nin, int cw, int c)
 {
-    const int e0 = c * a.cw, last = min(nin, e0 + a.cw) - 1 - e0;
+    const int e0 = c * cw, last = min(nin, e0 + cw) - 1 - e0;
     return ChunkEnds{chan_scales(cf, e0), chan_scales(cf, e0 + last)};
 }
 
@@ -473,12 +496,11 @@ __device__ int axis_step(float c32, const ChanF *cf, const ChanD *cd, int e0, in
 // scales at the chunk's two end channels).  The cell index is monotone in
 // frequency along each axis, so the cells at a chunk's two end channels
 // bound every channel between.
-__device__ int2 chunk_cell(const RunArgs &a, const SrcDev &S, const ChanF *cf, const ChanD *cd, int c, float uf,
-                           float vf, const double *uvw, bool fold, const ChunkEnds &ce)
+__device__ int2 chunk_cell(const RunArgs &a, const ChanF *cf, const ChanD *cd, int nin, int cw, int c, float uf, float vf,
+                           const double *uvw, bool fold, const ChunkEnds &ce)
 {
-    const int nin = S.k_hi - S.k_lo;
     const float hu = (float)(a.g.nu >> 1), hv = (float)(a.g.nv >> 1);
-    const int e0 = c * a.cw, last = min(nin, e0 + a.cw) - 1 - e0;
+    const int e0 = c * cw, last = min(nin, e0 + cw) - 1 - e0;
     const float fu0 = axis_floor(uf, ce.s0.x, uvw, fold, &cd[e0].su);
     const float fu1 = axis_floor(uf, ce.s1.x, uvw, fold, &cd[e0 + last].su);
     const float fv0 = axis_floor(vf, ce.s0.y, uvw + 1, fold, &cd[e0].sv);
@@ -593,13 +615,14 @@ __global__ void __launch_bounds__(256) k_rows(RunArgs a)
     const ChanD *cd = a.chd + S.chan_off;
     const ChanF *cf = a.chf + S.chan_off;
     int2 *out = a.ccells + S.cell_off + q;
-    const int nchunk = S.nchunk, nin = S.k_hi - S.k_lo;
+    const int nchunk = S.nchunk, nin = S.k_hi - S.k_lo, cw = S.cw;
+    const int64_t nrow = S.nrow;
     if (nchunk <= 0) return;
-    ChunkEnds nx = chunk_ends(a, cf, nin, 0);
+    ChunkEnds nx = chunk_ends(cf, nin, cw, 0);
     for (int c = 0; c < nchunk; ++c) {
         const ChunkEnds ce = nx;
-        if (c + 1 < nchunk) nx = chunk_ends(a, cf, nin, c + 1);
-        out[(int64_t)c * S.nrow] = chunk_cell(a, S, cf, cd, c, uf, vf, guvw, fold, ce);
+        if (c + 1 < nchunk) nx = chunk_ends(cf, nin, cw, c + 1);
+        out[c * nrow] = chunk_cell(a, cf, cd, nin, cw, c, uf, vf, guvw, fold, ce);
     }
 }
 

@@ -10,7 +10,8 @@
 //      streams) run while the wave before is stacked, two staging slots
 //      taking turns (the streaming pipeline of Sec. 3.1/3.3: read ->
 //      compute overlapped)
-//   5. per class: row ordering + records + work list, then the persistent
+//   5. per wave: row ordering + records + work lists of all its classes in one
+//      pre-pass, then each class's persistent
 //      stacking kernel (mixed or FP64)
 #include <algorithm>
 #include <cmath>
@@ -173,12 +174,12 @@ int choose_ns(int nin, int cap)
 
 inline size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Layout of the shared ordering buffer for one class.
+// Layout of the shared ordering buffer for one pre-pass.
 struct SortLayout {
     size_t hist, qstart, ioff, segcnt, slot, key, perm, tmp, items, ctr, total;
 };
 
-SortLayout sort_layout(int64_t rows, int64_t nbuckets, int64_t max_items, int64_t nseg, int nstripe)
+SortLayout sort_layout(int64_t rows, int64_t nbuckets, int64_t max_items, int64_t nseg, int nstripe, size_t nclass)
 {
     SortLayout L{};
     size_t o = 0;
@@ -201,30 +202,31 @@ SortLayout sort_layout(int64_t rows, int64_t nbuckets, int64_t max_items, int64_
     L.items = o;
     o += al256(sizeof(Item) * (size_t)max_items);
     L.ctr = o;
-    o += 256;
+    o += al256(4 * (nclass + 1));
     L.total = o;
     return L;
 }
 
-// One launch class: the row-ordering pre-pass and the stacking kernel.
-cudaError_t launch_class(vista_stack *h, const ClassRun &cr, cudaStream_t st)
+// The row-ordering pre-pass of a group of classes, then their stacking
+// kernels.  One pre-pass for all classes: its kernels are bound by latency,
+// not by the rows, when the classes are small (three classes of four windows
+// of a few thousand rows, kernel time: 204 us in three pre-passes, 93 in one).
+cudaError_t launch_group(vista_stack *h, const PrepRun &pr, cudaStream_t st)
 {
     const bool fp64 = h->desc.precision == VISTA_PREC_FP64;
     const LaunchCfg cfg = h->cfg;
-    cudaError_t e = cudaSuccess;
-    {
-        const RunArgs &a = cr.args;
-        int sp = span_begin(h, 0);
-        int nk = 0;
-        e = launch_prepare(a, st, &nk);
+    int sp = span_begin(h, 0);
+    int nk = 0;
+    cudaError_t e = launch_prepare(pr.args, st, &nk);
+    span_end(h, sp);
+    if (h->timing) h->tacc.launches += nk;
+    for (size_t ci = pr.c0; ci < pr.c1 && e == cudaSuccess; ++ci) {
+        const ClassRun &cr = h->classes[ci];
+        sp = span_begin(h, 1);
+        e = fp64 ? launch_fp64(cr.args, cr.key, st)
+                 : launch_mixed(cr.args, cr.key, cfg.warps_per_cta, cfg.prefetch_rows, st);
         span_end(h, sp);
-        if (h->timing) h->tacc.launches += nk;
-        if (e == cudaSuccess) {
-            sp = span_begin(h, 1);
-            e = fp64 ? launch_fp64(a, cr.key, st) : launch_mixed(a, cr.key, cfg.warps_per_cta, cfg.prefetch_rows, st);
-            span_end(h, sp);
-            if (h->timing) h->tacc.launches += 1;
-        }
+        if (h->timing) h->tacc.launches += 1;
     }
     return e;
 }
@@ -240,8 +242,8 @@ cudaError_t device_pass(vista_stack *h, cudaStream_t st)
                               st);
         if (e != cudaSuccess) return e;
     }
-    for (const ClassRun &cr : h->classes)
-        if ((e = launch_class(h, cr, st)) != cudaSuccess) return e;
+    for (const PrepRun &pr : h->preps)
+        if ((e = launch_group(h, pr, st)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -262,7 +264,7 @@ cudaError_t streamed_pass(vista_stack *h)
         e = cudaMemcpy2DAsync(cp.dst, cp.dpitch, cp.src, cp.spitch, cp.width, cp.height, cudaMemcpyDeviceToDevice,
                               h->stream);
     }
-    size_t ci = 0;
+    size_t pi = 0;
     for (int w = 0; w < h->nwaves && e == cudaSuccess; ++w) {
         const int slot = w & 1;
         for (int j = 0; j < NXFER && e == cudaSuccess && w >= 2; ++j)
@@ -277,8 +279,8 @@ cudaError_t streamed_pass(vista_stack *h)
                 e = cudaMemcpy2DAsync(c.dst, c.dpitch, c.src, c.spitch, c.width, c.height, cudaMemcpyHostToDevice, cs);
         }
         if (e == cudaSuccess) e = xfer_join(h);   // the stream waits for this wave's copies
-        while (e == cudaSuccess && ci < h->classes.size() && h->classes[ci].wave == w)
-            e = launch_class(h, h->classes[ci++], h->stream);
+        while (e == cudaSuccess && pi < h->preps.size() && h->classes[h->preps[pi].c0].wave == w)
+            e = launch_group(h, h->preps[pi++], h->stream);
         if (e == cudaSuccess) e = cudaEventRecord(h->slot_ev[slot], h->stream);
     }
     return e;
@@ -526,7 +528,6 @@ extern "C" int vista_run(vista_stack *h)
 
     std::vector<SrcDev> sdev;
     std::vector<double> rots;   // 9 per re-projected window (SrcDev::rot1 - 1 indexes them)
-    std::vector<char> cls_rot(classes.size(), 0);
     // gridding baselines of the re-projected windows (filled by k_keys)
     int64_t rot_rows = 0, guvw_pos = 0;
     for (const SrcHost &s : h->pending)
@@ -534,28 +535,37 @@ extern "C" int vista_run(vista_stack *h)
     if (rot_rows > 0 && (e = h->b_guvw.ensure((size_t)rot_rows * 24)) != cudaSuccess)
         return cuda_fail(h, e, "re-projection buffer allocation");
     std::vector<int64_t> offs;
-    std::vector<size_t> cls_src0(classes.size()), cls_off0(classes.size());
-    std::vector<SortLayout> layouts(classes.size());
+    // one pre-pass per wave: its classes' windows one after the other
+    std::vector<PrepRun> preps;
+    std::vector<size_t> prep_src0, prep_off0;
+    std::vector<SortLayout> layouts;
     size_t sort_bytes = 0;
+    const int nst = cfg.sort_rows ? h->nstripe : 1;
     int64_t rec_total = 0, cell_total = 0;
     uint64_t nvis_run = 0, bound_run = 0;
     std::vector<Copy2D> copies;
     std::vector<HostCopy> hcopies;
     std::vector<size_t> wave_pos((size_t)std::max(nwaves, 1), 0);   // next free byte of each wave's slot
     size_t stage_pos = host_region;                                  // the repacked flags follow the slots
-    for (size_t ci = 0; ci < classes.size(); ++ci) {
-        ClassRun &cr = classes[ci];
-        const int cw = 32 * cr.ns;
-        cls_src0[ci] = sdev.size();
-        cls_off0[ci] = offs.size();
-        const size_t m = cr.members.size();
+    for (size_t c0 = 0, c1; c0 < classes.size(); c0 = c1) {
+        std::vector<int> windows, width;   // the wave's windows, class by class, and their chunk widths
+        std::vector<int64_t> coff;
+        for (c1 = c0; c1 < classes.size() && classes[c1].wave == classes[c0].wave; ++c1) {
+            classes[c1].w0 = (int)windows.size();
+            coff.push_back((int64_t)windows.size());
+            windows.insert(windows.end(), classes[c1].members.begin(), classes[c1].members.end());
+            width.resize(windows.size(), 32 * classes[c1].ns);
+        }
+        const size_t m = windows.size();
+        coff.push_back((int64_t)m);
+        prep_src0.push_back(sdev.size());
+        prep_off0.push_back(offs.size());
         std::vector<int64_t> roff(m + 1, 0), soff(m + 1, 0);
-        int64_t max_items = 0, class_rows = 0;
-        for (int i : cr.members) class_rows += h->pending[(size_t)i].d.nrow;
-        const int seg = segment_rows(class_rows);
-        cr.args.so.seg_rows = seg;
+        int64_t max_items = 0, rows = 0;
+        for (int i : windows) rows += h->pending[(size_t)i].d.nrow;
+        const int seg = segment_rows(rows);
         for (size_t t = 0; t < m; ++t) {
-            const int i = cr.members[t];
+            const int i = windows[t], cw = width[t];
             const SrcHost &s = h->pending[(size_t)i];
             const Plan &pl = plans[(size_t)i];
             const int32_t nin = pl.k_hi - pl.k_lo;
@@ -632,6 +642,7 @@ extern "C" int vista_run(vista_stack *h)
             d.linear = pl.linear ? 1 : 0;
             for (int p = 0; p < 4; ++p) d.plane[p] = p < s.d.npol ? s.pol_map[(size_t)p] : -1;
             d.nchunk = (nin + cw - 1) / cw;
+            d.cw = cw;
             d.key_su = (float)(s.freqs[(size_t)pl.key_ch] * gu);
             d.key_sv = (float)(s.freqs[(size_t)pl.key_ch] * gv);
             d.rec_off = rec_total;
@@ -654,20 +665,24 @@ extern "C" int vista_run(vista_stack *h)
                 rots.insert(rots.end(), s.rot, s.rot + 9);
                 d.guvw = (const double *)h->b_guvw.p + 3 * guvw_pos;
                 guvw_pos += d.nrow;
-                cls_rot[ci] = 1;
             }
             sdev.push_back(d);
         }
         offs.insert(offs.end(), roff.begin(), roff.end());
         offs.insert(offs.end(), soff.begin(), soff.end());
-        cr.args.so.nseg_total = soff[m];
-        cr.args.nsrc = (int32_t)m;
-        cr.args.cw = cw;
-        cr.args.nrows_total = roff[m];
-        const int nst = cfg.sort_rows ? h->nstripe : 1;
-        layouts[ci] = sort_layout(roff[m], (int64_t)m * nst, max_items, soff[m], nst);
-        cr.args.so.max_items = max_items;
-        sort_bytes = std::max(sort_bytes, layouts[ci].total);
+        offs.insert(offs.end(), coff.begin(), coff.end());
+        PrepRun pr;
+        pr.c0 = c0;
+        pr.c1 = c1;
+        pr.args.nsrc = (int32_t)m;
+        pr.args.nrows_total = roff[m];
+        pr.args.so.seg_rows = seg;
+        pr.args.so.nseg_total = soff[m];
+        pr.args.so.max_items = max_items;
+        pr.args.so.nclass = (int32_t)(c1 - c0);
+        preps.push_back(pr);
+        layouts.push_back(sort_layout(roff[m], (int64_t)m * nst, max_items, soff[m], nst, c1 - c0));
+        sort_bytes = std::max(sort_bytes, layouts.back().total);
     }
 
     // uploads and buffers
@@ -693,17 +708,17 @@ extern "C" int vista_run(vista_stack *h)
 
     // 5. launch arguments, then the device pass
     const CubeGeom g{c.nu, c.nv, c.nrest, c.npol, gu, gv, c.hermitian_fold, 0};
-    for (size_t ci = 0; ci < classes.size(); ++ci) {
-        ClassRun &cr = classes[ci];
-        RunArgs &a = cr.args;
-        a.srcs = (const SrcDev *)h->b_srcs.p + cls_src0[ci];
+    for (size_t pi = 0; pi < preps.size(); ++pi) {
+        RunArgs &a = preps[pi].args;
+        a.srcs = (const SrcDev *)h->b_srcs.p + prep_src0[pi];
         a.chf = (const ChanF *)h->b_chf.p;
         a.chd = (const ChanD *)h->b_chd.p;
         a.recs = (RowRec *)h->b_recs.p;
-        a.rot = cls_rot[ci] ? (const double *)h->b_rot.p : nullptr;
+        a.rot = rots.empty() ? nullptr : (const double *)h->b_rot.p;
         a.ccells = (int2 *)h->b_cells.p;
-        a.row_off = (const int64_t *)h->b_off.p + cls_off0[ci];
-        a.so.seg_off = a.row_off + cr.members.size() + 1;
+        a.row_off = (const int64_t *)h->b_off.p + prep_off0[pi];
+        a.so.seg_off = a.row_off + a.nsrc + 1;
+        a.so.cls_off = a.so.seg_off + a.nsrc + 1;
         a.g = g;
         a.cube = h->cube;
         a.cube_master = h->cube_master;
@@ -712,7 +727,7 @@ extern "C" int vista_run(vista_stack *h)
         a.stats = h->stats;
         a.err = h->err;
         SortArgs &so = a.so;
-        const SortLayout &L = layouts[ci];
+        const SortLayout &L = layouts[pi];
         char *b = (char *)h->b_sort.p;
         so.hist = (uint32_t *)(b + L.hist);
         so.qstart = (uint32_t *)(b + L.qstart);
@@ -726,12 +741,18 @@ extern "C" int vista_run(vista_stack *h)
         so.ctr = (uint32_t *)(b + L.ctr);
         so.sorted = cfg.sort_rows;
         so.stripe_rows = cfg.sort_rows ? h->stripe_rows : c.nv;
-        so.nstripe = cfg.sort_rows ? h->nstripe : 1;
+        so.nstripe = nst;
         so.ushift = h->ushift;
         so.nuk = h->nuk;
         so.rows_per_item = cfg.rows_per_item;
+        for (size_t ci = preps[pi].c0; ci < preps[pi].c1; ++ci) {
+            classes[ci].args = a;
+            classes[ci].args.cls = (int32_t)(ci - preps[pi].c0);
+            classes[ci].args.cw = 32 * classes[ci].ns;
+        }
     }
     h->classes = std::move(classes);
+    h->preps = std::move(preps);
     h->copies = std::move(copies);
     h->hcopies = std::move(hcopies);
     h->nwaves = nwaves;

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(KMAX_THREADS, (min_blocks<P>())) stack_mixed(R
     }
     __syncwarp();
 
-    const uint32_t nitems = a.so.ctr[0];
+    const uint32_t nitems = a.so.ctr[a.cls + 1];   // end of the class's items
     const uint32_t G = gridDim.x * (blockDim.x >> 5);
     const uint32_t gw = blockIdx.x * (blockDim.x >> 5) + wid;
     const int npol_c = a.g.npol, nrest = a.g.nrest, gnu = a.g.nu, gnv = a.g.nv;
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(KMAX_THREADS, (min_blocks<P>())) stack_mixed(R
         tma_load_1d(S.cells, a.ccells + e0a, b_cc, &bars[s]);
     };
 
-    uint32_t it = gw;
+    uint32_t it = a.so.ctr[a.cls] + gw;
     if (lane == 0 && it < nitems) {
         const Item first = a.so.items[it];
         issue(0, it, first, it + G);
