@@ -287,10 +287,18 @@ __device__ __forceinline__ float2 subtract_fit(const EntryFF &v, float2 x, const
 // (exact products by FMA).  Entries whose count is 0 are zero: both passes
 // read the counts of CELL_UNROLL rows of 32 entries together and load only
 // the touched ones; `all` takes every entry as touched (counts that may have
-// wrapped, see cube_counts_exact()).  2.7e8 entries of four planes, 10 % of
-// the cells and 6.3 % of the entries touched, order 1: 3704 us when every
-// entry was read twice, 1142 us so (4.3 TB/s of the 4.9 GB moved).
-constexpr int CELL_UNROLL = 8;
+// wrapped, see cube_counts_exact()).  A cell is first looked over for any
+// touched entry, 16 bytes of counts a lane and WIDE_LOADS loads together
+// (`wide`: its entries are whole quadruples and the output is aligned), and
+// the blocks take the cells in an order that spreads neighbours (`spread`):
+// the touched ones lie together, and their warps, bound by latency, then run
+// beside others that stream.  2.7e8 entries of four planes, 10 % of the cells
+// and 6.3 % of the entries touched, order 1: 3704 us when every entry was read
+// twice, 1125 us in cell order with the counts a word at a time, 963 us so
+// (5.1 TB/s of the 4.9 GB moved; the second pass finds its entries evicted from
+// L2).  Slower: several warps a cell (1500 us: their FP64 reductions and
+// solves), entries of two or four rows loaded together (1780, 2460: registers).
+constexpr int CELL_UNROLL = 8, WIDE_LOADS = 8, CELL_THREADS = 128;
 
 // Bit q: entry base + 32 q + lane of the cell is touched.
 __device__ __forceinline__ uint32_t touched_bits(const uint32_t *cnt, int base, int lane, int nent, int all)
@@ -305,18 +313,40 @@ __device__ __forceinline__ uint32_t touched_bits(const uint32_t *cnt, int base, 
 }
 
 template <int ORDER>
-__global__ void __launch_bounds__(256) k_contsub_cell(const void *cube, const double *master, const uint32_t *count,
+__global__ void __launch_bounds__(CELL_THREADS) k_contsub_cell(const void *cube, const double *master, const uint32_t *count,
                                                       int fp64, int all, const uint8_t *line_free, int64_t ncell,
-                                                      int nrest, int lg_npol, float2 inv, float2 *out)
+                                                      int nrest, int lg_npol, int wide, uint32_t spread, float2 inv, float2 *out)
 {
     constexpr int NM = 2 * ORDER + 1;
     constexpr int NB = ORDER + 1;
     const int lane = threadIdx.x & 31, npol = 1 << lg_npol;
-    const int64_t cell = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t block = (int64_t)((uint64_t)blockIdx.x * spread % gridDim.x);
+    const int64_t cell = (block * blockDim.x + threadIdx.x) >> 5;
     if (cell >= ncell) return;   // whole warps
     const int64_t e0 = cell * nrest * npol;
     const int nent = nrest * npol;
     const uint32_t *cnt = count + e0;
+    if (wide) {   // is any entry touched?  16 bytes of counts a lane at a time
+        const uint4 *c4 = reinterpret_cast<const uint4 *>(cnt);
+        const int n4 = nent >> 2;
+        uint32_t any4 = 0u;
+        for (int i0 = 0; i0 < n4 && !__any_sync(0xffffffffu, any4 != 0u); i0 += 32 * WIDE_LOADS) {
+#pragma unroll
+            for (int k = 0; k < WIDE_LOADS; ++k) {
+                const int i = i0 + 32 * k + lane;
+                if (i < n4) {
+                    const uint4 c = __ldcs(c4 + i);
+                    any4 |= c.x | c.y | c.z | c.w;
+                }
+            }
+        }
+        if (!__any_sync(0xffffffffu, any4 != 0u)) {   // an untouched cell: no fit, all sums zero
+            float4 *o4 = reinterpret_cast<float4 *>(out + e0);
+#pragma unroll 4
+            for (int i = lane; i < nent / 2; i += 32) __stcs(o4 + i, make_float4(0.f, 0.f, 0.f, 0.f));
+            return;
+        }
+    }
     MomentsFF<ORDER> mo;
     mo.zero();
     int nfit = 0;
@@ -497,6 +527,24 @@ __global__ void __launch_bounds__(256) k_contsub(const void *cube, const double 
     }
 }
 
+// A stride that visits the blocks 0 ... n - 1 in an order which spreads
+// neighbours: near 0.618 n and without a common divisor with n.
+uint32_t block_spread(uint32_t n)
+{
+    uint32_t s = (uint32_t)(0.6180339887 * n);
+    auto gcd = [](uint32_t a, uint32_t b) {
+        while (b) {
+            const uint32_t t = a % b;
+            a = b;
+            b = t;
+        }
+        return a;
+    };
+    if (s == 0) s = 1;
+    while (gcd(s, n) != 1) ++s;
+    return s;
+}
+
 cudaError_t launch_contsub(const vista_stack *h, const uint8_t *line_free, int order, float2 *out, cudaStream_t st)
 {
     const int64_t ncell = (int64_t)h->desc.nu * h->desc.nv;
@@ -508,12 +556,14 @@ cudaError_t launch_contsub(const vista_stack *h, const uint8_t *line_free, int o
         const int all = cube_counts_exact(h) ? 0 : 1, lg = npol == 4 ? 2 : npol == 2 ? 1 : 0;
         const double r = 1.0 / (double)nrest;
         const float2 inv = make_float2((float)r, (float)(r - (double)(float)r));
-        const unsigned cb = (unsigned)((ncell * 32 + 255) / 256);
+        const unsigned cb = (unsigned)((ncell * 32 + CELL_THREADS - 1) / CELL_THREADS);
+        const int wide = !all && (nrest * npol) % 4 == 0 && ((uintptr_t)out & 15) == 0;
+        const uint32_t spread = block_spread(cb);
         switch (order) {
-        case 0: k_contsub_cell<0><<<cb, 256, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, inv, out); break;
-        case 1: k_contsub_cell<1><<<cb, 256, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, inv, out); break;
-        case 2: k_contsub_cell<2><<<cb, 256, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, inv, out); break;
-        case 3: k_contsub_cell<3><<<cb, 256, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, inv, out); break;
+        case 0: k_contsub_cell<0><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
+        case 1: k_contsub_cell<1><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
+        case 2: k_contsub_cell<2><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
+        case 3: k_contsub_cell<3><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
         default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
