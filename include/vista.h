@@ -82,10 +82,9 @@ typedef struct vista_stack vista_stack;   /* opaque handle */
  *              body, an FP32 cube whose entries are moved into an FP64 master
  *              cube at checkpoints spread over the drains and folded into it
  *              wholly after a run once 64 visibilities per cube entry have
- *              been stacked since the last fold (measured within 4.3e-6
- *              relative on every entry of a 3.8e11-visibility stack, and the
- *              same after stacking it twice); VISTA_PREC_FP64: the plain
- *              form, FP64 throughout with an FP64 cube.
+ *              been stacked since the last fold (measured within 6e-7
+ *              relative on every entry of a 1.9e11-visibility stack stacked
+ *              twice); VISTA_PREC_FP64: FP64 throughout with an FP64 cube.
  *   hermitian_fold  1: rows with v < 0 (or v == 0, u < 0) are negated and
  *              their shifted visibility conjugated before binning.
  *   stream     cudaStream_t for all device work (NULL = legacy default stream). */
@@ -156,7 +155,7 @@ typedef struct {
 
 /* Launch shape of the mixed-precision path (0 fields = library default).
  *   rows_per_item   rows one warp walks through per work item (1..256; their
- *                   FP64 records are staged in shared memory).
+ *                   records are staged in shared memory).
  *   chans_per_lane  channels per lane in one item (item = 32 x this many
  *                   channels; 1, 2 or 4).
  *   warps_per_cta   warps per block of the stacking kernel.
@@ -225,12 +224,9 @@ int vista_add_source_reproject(vista_stack *h, const vista_source_desc *src, dou
  * device arrays of nrow x nrest x npol entries, owned by the caller.  Each
  * row's delay is formed in FP64 and kept as a float-float pair; each
  * contributor's phasor comes from a float-float phase (error below 5e-7 rad)
- * and the sums are FP32.  One thread per (row, output channel); synchronous
- * on the handle's stream.  The cube and the queue are not touched.
- * Alignment changes only the speed: complex64 vis with 2 or 4 pols on a
- * 16-byte boundary is read in vector loads, and with 2 or 4 pols, out_vis
- * on a 16-byte and out_wsum on a 16-byte (4 pols) or 8-byte (2 pols)
- * boundary are written in vector stores.
+ * and the sums are FP32.  Synchronous on the handle's stream.  The cube and
+ * the queue are not touched.  Alignment changes only the speed (out_vis on an
+ * 8-byte boundary: a value's two floats are written in one store).
  * E_STATE: the lattice is not fixed yet (open with rest_df > 0, or run
  * first).  E_ARG: a host-visible field fails the checks of vista_add_source
  * (nchan >= 2 here). */

@@ -18,8 +18,9 @@
 //
 // Before (a thread per row, every visibility's bins written by FP64 atomics)
 // and now, kernel time: 1.7e7 visibilities of two pols in complex128, 1254 ->
-// 653 us (and 124 us of pre-pass it did without); 3.5e7 of four pols, 3732 ->
-// 1023 us; 8.7e6 of one pol, 739 -> 378 us.  The FP64 pipe is 81 % busy.
+// 590 us (and about 80 us of pre-pass it did without); 3.5e7 of four pols, 3732
+// -> 1023 us and 8.7e6 of one pol, 739 -> 378 us, both before the rows of a cell
+// were ordered by parts (653 us then for two pols).  The FP64 pipe is 81 % busy.
 #include "vista_device.cuh"
 
 namespace vista {

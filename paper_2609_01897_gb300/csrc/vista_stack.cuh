@@ -21,8 +21,9 @@
 // L2 twice); the warp then synchronises before a group's values are read and
 // before their ring slots are refilled.
 //
-// The kernel is bound by instruction issue before it is bound by HBM, so it
-// is built to spend few instructions per (row, 32 channels):
+// The kernel is bound by the issue and latency of its instructions (57 to 62 %
+// issue with 15 warps an SM) before it is bound by HBM, so it is built to spend
+// few instructions per (row, 32 channels):
 //  - the arithmetic is in packed FP32 pairs (one instruction per pair): with
 //    (c, s) the phasor and v = (re, im) a value, the sums of W v c and W v s
 //    are kept as pairs and combined (re = C.re - S.im, im = C.im + S.re) only
@@ -45,15 +46,16 @@
 // 2.2e11 32-byte sectors of reductions a second however few of their bytes
 // change, and does not combine lanes of one address, so without the merging
 // the reductions bound the kernel (0.49 of them per visibility on a compact
-// array's stack, 0.28 merged; 0.150 and 0.022 on an archive stack).  Runs off
-// the grid only feed the dropped counter.
+// array's stack, 0.25 merged; 0.150 and 0.019 on an archive stack; without any
+// the kernel would now gain 1 to 2 %).  Runs off the grid only feed the dropped
+// counter.
 //
 // Measured, before (values through predicated scalar arithmetic, one row at a
 // time, runs written unmerged) and now, kernel time: a compact array's stack,
-// two pols of complex64, 5.2e8 visibilities, 1.96 -> 1.67 ms; an archive
-// stack, 1.2e10 visibilities of two and four pols, 28.5 -> 23.6 ms (4.7 TB/s);
-// wideband FP16, 7.5e8 visibilities, 2.75 -> 2.24 ms; long baselines in BF16,
-// 4.6e8 visibilities, 1.46 -> 1.19 ms.  Per (row, 32 channels) of two pols a
+// two pols of complex64, 5.2e8 visibilities, 1.96 -> 1.61 ms; an archive
+// stack, 1.2e10 visibilities of two and four pols, 28.5 -> 23.2 ms (4.8 TB/s);
+// wideband FP16, 7.5e8 visibilities, 2.75 -> 1.90 ms; long baselines in BF16,
+// 4.6e8 visibilities, 1.46 -> 1.14 ms.  Per (row, 32 channels) of two pols a
 // warp issues about 78 instructions where no run ends (99 before the row loop
 // lost its branches), 112 on the compact array's stack (178 before).
 #pragma once
