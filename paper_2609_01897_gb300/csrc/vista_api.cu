@@ -225,6 +225,8 @@ extern "C" int vista_open_stack(const vista_cube_desc *d, vista_stack **out)
     if (e == cudaSuccess) e = cudaMemsetAsync(h->cube, 0, (size_t)n * esz, h->stream);
     if (e == cudaSuccess && !fp64c) e = cudaMalloc((void **)&h->cube_master, (size_t)n * 32);
     if (e == cudaSuccess && !fp64c) e = cudaMemsetAsync(h->cube_master, 0, (size_t)n * 32, h->stream);
+    if (e == cudaSuccess && !fp64c) e = cudaMalloc((void **)&h->moved, moved_bytes(n));
+    if (e == cudaSuccess && !fp64c) e = cudaMemsetAsync(h->moved, 0, moved_bytes(n), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->count, 0, (size_t)n * sizeof(uint32_t), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->stats, 0, sizeof(DevStats), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int32_t), h->stream);
@@ -233,6 +235,7 @@ extern "C" int vista_open_stack(const vista_cube_desc *d, vista_stack **out)
         const int rc = cuda_fail(nullptr, e, "cube allocation");
         cudaFree(h->cube);
         cudaFree(h->cube_master);
+        cudaFree(h->moved);
         cudaFree(h->count);
         cudaFree(h->stats);
         cudaFree(h->err);
@@ -388,7 +391,7 @@ int read_common(vista_stack *h, void *sum_wv, void *sum_w, void *sum_wvv, uint32
     const int64_t n = h->nentries;
     const size_t fe = out_f64 ? 8 : 4;
     if (dst_dev) {
-        e = launch_unpack(h->cube, h->cube_master, h->count, fp64, all, n, sum_wv, sum_w, sum_wvv, count, out_f64,
+        e = launch_unpack(h->cube, h->cube_master, h->moved, h->count, fp64, all, n, sum_wv, sum_w, sum_wvv, count, out_f64,
                           h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "cube unpack");
         return finish_with_error_word(h, "cube unpack");
@@ -403,7 +406,7 @@ int read_common(vista_stack *h, void *sum_wv, void *sum_w, void *sum_wvv, uint32
     char *d_w = sum_w ? p + b_wv : nullptr;
     char *d_vv = sum_wvv ? p + b_wv + b_w : nullptr;
     uint32_t *d_c = count ? (uint32_t *)(p + b_wv + b_w + b_vv) : nullptr;
-    e = launch_unpack(h->cube, h->cube_master, h->count, fp64, all, n, d_wv, d_w, d_vv, d_c, out_f64, h->stream);
+    e = launch_unpack(h->cube, h->cube_master, h->moved, h->count, fp64, all, n, d_wv, d_w, d_vv, d_c, out_f64, h->stream);
     // the four arrays go back on the copy streams, in parallel
     if (e == cudaSuccess) e = xfer_fork(h);
     if (e == cudaSuccess && sum_wv) e = cudaMemcpyAsync(sum_wv, d_wv, b_wv, cudaMemcpyDeviceToHost, h->xfer[0]);
@@ -459,7 +462,7 @@ extern "C" int vista_read_cube_async(vista_stack *h, float *sum_wv, float *sum_w
     // follows the runs queued so far on the handle's stream
     if (h->rb_pending) e = cudaStreamWaitEvent(h->stream, h->rb_done, 0);
     if (e == cudaSuccess)
-        e = launch_unpack(h->cube, h->cube_master, h->count, fp64, all, n, d_wv, d_w, d_vv, d_c, 0, h->stream);
+        e = launch_unpack(h->cube, h->cube_master, h->moved, h->count, fp64, all, n, d_wv, d_w, d_vv, d_c, 0, h->stream);
     if (e == cudaSuccess) e = cudaEventRecord(h->rb_ready, h->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->rb_stream, h->rb_ready, 0);
     if (e == cudaSuccess && sum_wv) e = cudaMemcpyAsync(sum_wv, d_wv, b_wv, cudaMemcpyDeviceToHost, h->rb_stream);
@@ -517,7 +520,7 @@ extern "C" int vista_read_cube_sparse(vista_stack *h, int64_t cap, int64_t *inde
         return fail(h, VISTA_E_RANGE, "the cube has %lld touched entries, more than cap = %lld", (long long)total,
                     (long long)cap);
     if (dst_is_device) {
-        e = launch_sparse_write(h->cube, h->cube_master, h->count, fp64, n, (const int64_t *)(b + o_off), cap, index,
+        e = launch_sparse_write(h->cube, h->cube_master, h->moved, h->count, fp64, n, (const int64_t *)(b + o_off), cap, index,
                                 sum_wv, sum_w, sum_wvv, count, h->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "sparse readback");
@@ -529,7 +532,7 @@ extern "C" int vista_read_cube_sparse(vista_stack *h, int64_t cap, int64_t *inde
                  need = o_c + al(t * 4);
     if ((e = h->b_unpack.ensure(need)) != cudaSuccess) return cuda_fail(h, e, "readback scratch allocation");
     char *u = (char *)h->b_unpack.p;
-    e = launch_sparse_write(h->cube, h->cube_master, h->count, fp64, n, (const int64_t *)(b + o_off), cap,
+    e = launch_sparse_write(h->cube, h->cube_master, h->moved, h->count, fp64, n, (const int64_t *)(b + o_off), cap,
                             (int64_t *)u, sum_wv ? (float *)(u + o_wv) : nullptr, sum_w ? (float *)(u + o_w) : nullptr,
                             sum_wvv ? (float *)(u + o_vv) : nullptr, count ? (uint32_t *)(u + o_c) : nullptr,
                             h->stream);
@@ -579,11 +582,12 @@ extern "C" int vista_zero_cube(vista_stack *h)
     const bool fp64 = h->desc.precision == VISTA_PREC_FP64;
     cudaError_t e;
     if (cube_counts_exact(h)) {
-        e = launch_zero_touched(h->cube, h->cube_master, h->count, h->stats, fp64, h->nentries, h->stream);
+        e = launch_zero_touched(h->cube, h->cube_master, h->moved, h->count, h->stats, fp64, h->nentries, h->stream);
     } else {
         e = cudaMemsetAsync(h->cube, 0, (size_t)h->nentries * (fp64 ? 32 : 16), h->stream);
         if (e == cudaSuccess && h->cube_master)
             e = cudaMemsetAsync(h->cube_master, 0, (size_t)h->nentries * 32, h->stream);
+        if (e == cudaSuccess && h->moved) e = cudaMemsetAsync(h->moved, 0, moved_bytes(h->nentries), h->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(h->count, 0, (size_t)h->nentries * 4, h->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(h->stats, 0, sizeof(DevStats), h->stream);
     }
@@ -755,6 +759,7 @@ extern "C" int vista_close(vista_stack *h)
     if (h->rb_done) cudaEventDestroy(h->rb_done);
     cudaFree(h->cube);
     cudaFree(h->cube_master);
+    cudaFree(h->moved);
     cudaFree(h->count);
     cudaFree(h->stats);
     cudaFree(h->err);

@@ -35,7 +35,8 @@ constexpr int MAX_ORDER = 3;
 
 // The entry's (sum_wv.re, sum_wv.im, sum_w) in FP64: the FP64 cube, or the
 // mixed path's FP32 partial plus its FP64 master.
-__device__ __forceinline__ double3 entry_sums(const void *cube, const double *master, int fp64, int64_t e)
+__device__ __forceinline__ double3 entry_sums(const void *cube, const double *master, const uint32_t *moved, int fp64,
+                                              int64_t e)
 {
     if (fp64) {
         const double *c = reinterpret_cast<const double *>(cube) + 4 * e;
@@ -43,7 +44,7 @@ __device__ __forceinline__ double3 entry_sums(const void *cube, const double *ma
     }
     const float4 f = reinterpret_cast<const float4 *>(cube)[e];
     double3 r = make_double3(f.x, f.y, f.z);
-    if (master) {
+    if (master && is_moved(moved[e >> 5], e)) {
         const double *m = master + 4 * e;
         r.x += m[0];
         r.y += m[1];
@@ -156,7 +157,7 @@ __device__ __forceinline__ float2 ff_of(double d)   // once per fit: FP64 conver
 struct EntryFF {
     float2 x, y, z;
 };
-__device__ __forceinline__ EntryFF entry_ff(const void *cube, const double *master, int fp64, int64_t e)
+__device__ __forceinline__ EntryFF entry_ff(const void *cube, const double *master, bool has_master, int fp64, int64_t e)
 {
     EntryFF r;
     if (fp64) {
@@ -168,7 +169,8 @@ __device__ __forceinline__ EntryFF entry_ff(const void *cube, const double *mast
     }
     const float4 f = reinterpret_cast<const float4 *>(cube)[e];
     if (master) {
-        const Double4 m = load_double4(master + 4 * e);
+        Double4 m{0.0, 0.0, 0.0, 0.0};
+        if (has_master) m = load_double4(master + 4 * e);
         r.x = add_ff(split_double(m.x), f.x);
         r.y = add_ff(split_double(m.y), f.y);
         r.z = add_ff(split_double(m.z), f.z);
@@ -312,8 +314,20 @@ __device__ __forceinline__ uint32_t touched_bits(const uint32_t *cnt, int base, 
     return t;
 }
 
+// Bit q: the master of entry e + 32 q, touched (t), may be nonzero.
+__device__ __forceinline__ uint32_t moved_bits(const uint32_t *moved, int64_t e, uint32_t t)
+{
+    uint32_t m = 0;
+    if (moved) {
+#pragma unroll
+        for (int q = 0; q < CELL_UNROLL; ++q)
+            if (((t >> q) & 1u) && is_moved(moved[(e + 32 * q) >> 5], e + 32 * q)) m |= 1u << q;
+    }
+    return m;
+}
+
 template <int ORDER>
-__global__ void __launch_bounds__(CELL_THREADS) k_contsub_cell(const void *cube, const double *master, const uint32_t *count,
+__global__ void __launch_bounds__(CELL_THREADS) k_contsub_cell(const void *cube, const double *master, const uint32_t *moved, const uint32_t *count,
                                                       int fp64, int all, const uint8_t *line_free, int64_t ncell,
                                                       int nrest, int lg_npol, int wide, uint32_t spread, float2 inv, float2 *out)
 {
@@ -354,6 +368,7 @@ __global__ void __launch_bounds__(CELL_THREADS) k_contsub_cell(const void *cube,
     uint32_t any = 0;
     for (int base = 0; base < nent; base += 32 * CELL_UNROLL) {
         const uint32_t t = touched_bits(cnt, base, lane, nent, all);
+        const uint32_t mv = moved_bits(moved, e0 + base + lane, t);
         uint32_t rows = __reduce_or_sync(0xffffffffu, t);
         any |= rows;
         while (rows) {
@@ -361,7 +376,7 @@ __global__ void __launch_bounds__(CELL_THREADS) k_contsub_cell(const void *cube,
             rows &= rows - 1u;
             const int f = base + 32 * q + lane, j = f >> lg_npol;
             if (!((t >> q) & 1u) || !line_free[j]) continue;
-            const EntryFF v = entry_ff(cube, master, fp64, e0 + f);
+            const EntryFF v = entry_ff(cube, master, (mv >> q) & 1u, fp64, e0 + f);
             if (!(v.z.x > 0.f)) continue;
             ++nfit;
             const float2 x = absc_ff(j, nrest, inv);
@@ -403,7 +418,7 @@ __global__ void __launch_bounds__(CELL_THREADS) k_contsub_cell(const void *cube,
         for (int f = lane; refine && f < nent; f += 32) {
             const int j = f >> lg_npol;
             if (!line_free[j] || (!all && cnt[f] == 0u)) continue;
-            const double3 v = entry_sums(cube, master, fp64, e0 + f);
+            const double3 v = entry_sums(cube, master, moved, fp64, e0 + f);
             if (!(v.z > 0.0)) continue;
             add_moments_fp64<ORDER>(v, (double)(2 * j - (nrest - 1)) * inv_n, Md, Brd, Bid);
         }
@@ -443,6 +458,7 @@ __global__ void __launch_bounds__(CELL_THREADS) k_contsub_cell(const void *cube,
     const int full = all || !__all_sync(0xffffffffu, finite);
     for (int base = 0; base < nent; base += 32 * CELL_UNROLL) {
         const uint32_t t = touched_bits(cnt, base, lane, nent, full);
+        const uint32_t mv = moved_bits(moved, e0 + base + lane, t);
         const uint32_t rows = __reduce_or_sync(0xffffffffu, t);
         for (int q = 0; q < CELL_UNROLL; ++q) {
             const int f = base + 32 * q + lane;
@@ -450,14 +466,14 @@ __global__ void __launch_bounds__(CELL_THREADS) k_contsub_cell(const void *cube,
             float2 o = make_float2(0.f, 0.f);
             if ((rows >> q) & 1u)
                 if ((t >> q) & 1u)
-                    o = subtract_fit<NB>(entry_ff(cube, master, fp64, e0 + f), absc_ff(f >> lg_npol, nrest, inv), fr, fi);
+                    o = subtract_fit<NB>(entry_ff(cube, master, (mv >> q) & 1u, fp64, e0 + f), absc_ff(f >> lg_npol, nrest, inv), fr, fi);
             out[e0 + f] = o;
         }
     }
 }
 
 template <int ORDER>
-__global__ void __launch_bounds__(256) k_contsub(const void *cube, const double *master, int fp64,
+__global__ void __launch_bounds__(256) k_contsub(const void *cube, const double *master, const uint32_t *moved, int fp64,
                                                  const uint8_t *line_free, int64_t ncell, int nrest, int npol,
                                                  float2 *out)
 {
@@ -480,7 +496,7 @@ __global__ void __launch_bounds__(256) k_contsub(const void *cube, const double 
     int nfit = 0;
     for (int j = lane; j < nrest; j += 32) {
         if (!line_free[j]) continue;
-        const double3 s = entry_sums(cube, master, fp64, entry(j));
+        const double3 s = entry_sums(cube, master, moved, fp64, entry(j));
         if (!(s.z > 0.0)) continue;
         ++nfit;
         const double x = absc(j);
@@ -515,7 +531,7 @@ __global__ void __launch_bounds__(256) k_contsub(const void *cube, const double 
 
     for (int j = lane; j < nrest; j += 32) {
         const int64_t e = entry(j);
-        const double3 s = entry_sums(cube, master, fp64, e);
+        const double3 s = entry_sums(cube, master, moved, fp64, e);
         const double x = absc(j);
         double pr = 0.0, pi = 0.0;
 #pragma unroll
@@ -560,10 +576,10 @@ cudaError_t launch_contsub(const vista_stack *h, const uint8_t *line_free, int o
         const int wide = !all && (nrest * npol) % 4 == 0 && ((uintptr_t)out & 15) == 0;
         const uint32_t spread = block_spread(cb);
         switch (order) {
-        case 0: k_contsub_cell<0><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
-        case 1: k_contsub_cell<1><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
-        case 2: k_contsub_cell<2><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
-        case 3: k_contsub_cell<3><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
+        case 0: k_contsub_cell<0><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->moved, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
+        case 1: k_contsub_cell<1><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->moved, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
+        case 2: k_contsub_cell<2><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->moved, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
+        case 3: k_contsub_cell<3><<<cb, CELL_THREADS, 0, st>>>(h->cube, m, h->moved, h->count, fp64, all, line_free, ncell, nrest, lg, wide, spread, inv, out); break;
         default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
@@ -571,10 +587,10 @@ cudaError_t launch_contsub(const vista_stack *h, const uint8_t *line_free, int o
     const int64_t warps = ncell * h->desc.npol;
     const unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
     switch (order) {
-    case 0: k_contsub<0><<<blocks, 256, 0, st>>>(h->cube, m, fp64, line_free, ncell, h->desc.nrest, h->desc.npol, out); break;
-    case 1: k_contsub<1><<<blocks, 256, 0, st>>>(h->cube, m, fp64, line_free, ncell, h->desc.nrest, h->desc.npol, out); break;
-    case 2: k_contsub<2><<<blocks, 256, 0, st>>>(h->cube, m, fp64, line_free, ncell, h->desc.nrest, h->desc.npol, out); break;
-    case 3: k_contsub<3><<<blocks, 256, 0, st>>>(h->cube, m, fp64, line_free, ncell, h->desc.nrest, h->desc.npol, out); break;
+    case 0: k_contsub<0><<<blocks, 256, 0, st>>>(h->cube, m, h->moved, fp64, line_free, ncell, h->desc.nrest, h->desc.npol, out); break;
+    case 1: k_contsub<1><<<blocks, 256, 0, st>>>(h->cube, m, h->moved, fp64, line_free, ncell, h->desc.nrest, h->desc.npol, out); break;
+    case 2: k_contsub<2><<<blocks, 256, 0, st>>>(h->cube, m, h->moved, fp64, line_free, ncell, h->desc.nrest, h->desc.npol, out); break;
+    case 3: k_contsub<3><<<blocks, 256, 0, st>>>(h->cube, m, h->moved, fp64, line_free, ncell, h->desc.nrest, h->desc.npol, out); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -25,6 +25,12 @@ __device__ __forceinline__ void store_zero32(void *p)
     asm volatile("st.global.v4.b64 [%0], {%1, %1, %1, %1};" ::"l"(p), "l"(0ll) : "memory");
 }
 
+// The mixed cube's master entries are zero but for those that a checkpoint or a
+// fold has moved sums into (about one touched entry in eight after a stack of six
+// reductions an entry); a bit per entry says which may not be, so that the other
+// masters' 32 bytes are neither read nor zeroed.
+__device__ __forceinline__ bool is_moved(uint32_t word, int64_t i) { return (word >> (i & 31)) & 1u; }
+
 // A double as hi + lo, two floats: hi is the double truncated to 24
 // significant bits, lo the remaining 29 bits rounded to a float (so hi + lo
 // is the double to about 2^-47 relative, less where lo falls below the

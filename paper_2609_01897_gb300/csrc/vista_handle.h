@@ -97,6 +97,7 @@ struct vista_stack {
     std::vector<vista::SrcHost> pending, last;
     void *cube = nullptr;
     double *cube_master = nullptr;   // mixed: FP64 sums moved out of the float4 cube at checkpoints
+    uint32_t *moved = nullptr;       // mixed: a bit per entry whose master may be nonzero
     uint32_t *count = nullptr;
     int64_t nentries = 0;
     vista::DevStats *stats = nullptr;

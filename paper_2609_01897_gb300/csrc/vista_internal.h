@@ -242,6 +242,7 @@ struct RunArgs {
     void *cube;                 // per entry: FP64 double[4], or float4 (mixed)
     double *cube_master;        // mixed with comp = 1: FP64 double[4] per entry, the sums moved
                                 // out of the float4 entries at checkpoints (value = master + float4)
+    uint32_t *moved;            // a bit per entry whose master may be nonzero (all others are zero)
     int32_t comp;
     uint32_t *count;
     DevStats *stats;
@@ -258,14 +259,15 @@ cudaError_t launch_mixed(const RunArgs &a, int key, int warps_per_cta, int prefe
 // The FP64 stacking kernel of one class (chunks of 32 channels), same key.
 cudaError_t launch_fp64(const RunArgs &a, int key, cudaStream_t st);
 // Mixed cube: move every FP32 partial into the FP64 master and clear it.
-cudaError_t launch_fold(void *cube, double *master, int64_t n, cudaStream_t st);
+inline size_t moved_bytes(int64_t n) { return (size_t)((n + 31) / 32) * sizeof(uint32_t); }
+cudaError_t launch_fold(void *cube, double *master, uint32_t *moved, int64_t n, cudaStream_t st);
 // Cube -> caller arrays; all = 1 reads every entry's sums, also where its count is 0.
-cudaError_t launch_unpack(const void *cube, const double *master, const uint32_t *count, int fp64, int all, int64_t n,
-                          void *sum_wv, void *sum_w, void *sum_wvv, uint32_t *cnt_out,
+cudaError_t launch_unpack(const void *cube, const double *master, const uint32_t *moved, const uint32_t *count, int fp64,
+                          int all, int64_t n, void *sum_wv, void *sum_w, void *sum_wvv, uint32_t *cnt_out,
                           int out_f64, cudaStream_t st);
 // Zero the entries whose count is not 0 (all others must be zero) and the counters.
-cudaError_t launch_zero_touched(void *cube, double *master, uint32_t *count, DevStats *stats, int fp64, int64_t n,
-                                cudaStream_t st);
+cudaError_t launch_zero_touched(void *cube, double *master, uint32_t *moved, uint32_t *count, DevStats *stats, int fp64,
+                                int64_t n, cudaStream_t st);
 // Sparse readback (the entries with count > 0, in entry order): per tile of
 // 4096 entries the touched count (tile_cnt [ntile]), their exclusive scan
 // (tile_off [ntile]) and the total (one int64 on the device); then each
@@ -274,7 +276,8 @@ cudaError_t launch_zero_touched(void *cube, double *master, uint32_t *count, Dev
 inline int64_t sparse_tiles(int64_t n) { return (n + 4095) / 4096; }
 cudaError_t launch_sparse_count(const uint32_t *count, int64_t n, uint32_t *tile_cnt, int64_t *tile_off,
                                 int64_t *total, cudaStream_t st);
-cudaError_t launch_sparse_write(const void *cube, const double *master, const uint32_t *count, int fp64, int64_t n,
+cudaError_t launch_sparse_write(const void *cube, const double *master, const uint32_t *moved, const uint32_t *count,
+                                int fp64, int64_t n,
                                 const int64_t *tile_off, int64_t cap, int64_t *index, float *sum_wv, float *sum_w,
                                 float *sum_wvv, uint32_t *cnt_out, cudaStream_t st);
 cudaError_t launch_debug(const RunArgs &a, int ns, int src, int fp64, double *ph, int32_t *cells,

@@ -105,12 +105,12 @@ struct RawEntry {
     float4 f;
     Double4 d;
 };
-__device__ __forceinline__ RawEntry load_entry(const void *cube, const double *master, int fp64, int64_t i)
+__device__ __forceinline__ RawEntry load_entry(const void *cube, const double *master, bool has_master, int fp64, int64_t i)
 {
     RawEntry r{make_float4(0.f, 0.f, 0.f, 0.f), Double4{0.0, 0.0, 0.0, 0.0}};
     if (!fp64) r.f = reinterpret_cast<const float4 *>(cube)[i];
-    const double *d = fp64 ? reinterpret_cast<const double *>(cube) : master;
-    if (d) r.d = load_double4(d + 4 * i);
+    if (fp64) r.d = load_double4(reinterpret_cast<const double *>(cube) + 4 * i);
+    else if (has_master) r.d = load_double4(master + 4 * i);
     return r;
 }
 template <typename T>
@@ -145,21 +145,38 @@ __device__ __forceinline__ void entry_value(const RawEntry &r, int fp64, T (&e)[
 // block apart, so that every access of a warp is contiguous and the counts of
 // all of them are in flight together.  Before (every entry read, widened,
 // added and narrowed on the FP64 pipe, which bound it) and now: 6.7e7 entries,
-// 31 % touched, 1478 -> 485 us (5.4 TB/s of the 2.6 GB it moves); 2.7e8
-// entries, 2.6 % touched, 5902 -> 1355 us (5.0 TB/s); 4.2e6 entries, 10 %
-// touched, 96 -> 23 us.
+// 31 % touched, 1478 -> 443 us (468 with the masters that are zero read too);
+// 2.7e8 entries, 2.6 % touched, 5902 -> 1365 us; 4.2e6 entries, 10 % touched, 96
+// -> 23 us.  It is at the rate of its writes: streaming stores, 16-byte stores of
+// four entries a thread and eight entries a thread were level or slower.
 constexpr int CUBE_THREADS = 256, CUBE_UNROLL = 4, CUBE_TILE = CUBE_THREADS * CUBE_UNROLL;
+constexpr int ZERO_UNROLL = 8, ZERO_TILE = CUBE_THREADS * ZERO_UNROLL;
+
+// The words of moved bits of a warp's entries b, b + CUBE_THREADS, ...: lane q
+// loads that of the q-th 32 entries, to be passed round by shuffles.
+__device__ __forceinline__ int64_t moved_at(int64_t b)
+{
+    const int lane = threadIdx.x & 31;
+    return (b - lane + (int64_t)lane * CUBE_THREADS) >> 5;
+}
+template <int N>
+__device__ __forceinline__ uint32_t moved_word(const uint32_t *moved, int64_t b, int64_t n)
+{
+    const int64_t w = moved_at(b);
+    return moved && (threadIdx.x & 31) < N && 32 * w < n ? moved[w] : 0u;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(CUBE_THREADS) unpack_kernel(const void *cube, const double *master,
-                                                              const uint32_t *count, int fp64, int all, int pair,
+                                                              const uint32_t *moved, const uint32_t *count, int fp64, int all, int pair,
                                                               int64_t n, T *sum_wv, T *sum_w, T *sum_wvv,
                                                               uint32_t *cnt_out)
 {
     struct alignas(2 * sizeof(T)) Pair {
         T re, im;
     };
-    for (int64_t b = (int64_t)blockIdx.x * CUBE_TILE + threadIdx.x; b < n; b += (int64_t)gridDim.x * CUBE_TILE) {
+    for (int64_t b0 = (int64_t)blockIdx.x * CUBE_TILE; b0 < n; b0 += (int64_t)gridDim.x * CUBE_TILE) {
+        const int64_t b = b0 + threadIdx.x;
         uint32_t c[CUBE_UNROLL];
         RawEntry r[CUBE_UNROLL];
 #pragma unroll
@@ -167,10 +184,12 @@ __global__ void __launch_bounds__(CUBE_THREADS) unpack_kernel(const void *cube, 
             const int64_t i = b + q * CUBE_THREADS;
             c[q] = i < n ? count[i] : 0u;
         }
+        const uint32_t word = moved_word<CUBE_UNROLL>(moved, b, n);
 #pragma unroll
         for (int q = 0; q < CUBE_UNROLL; ++q) {
             const int64_t i = b + q * CUBE_THREADS;
-            if (i < n && (all || c[q] != 0u)) r[q] = load_entry(cube, master, fp64, i);
+            const uint32_t mv = __shfl_sync(0xffffffffu, word, q);
+            if (i < n && (all || c[q] != 0u)) r[q] = load_entry(cube, master, is_moved(mv, i), fp64, i);
         }
 #pragma unroll
         for (int q = 0; q < CUBE_UNROLL; ++q) {
@@ -192,30 +211,37 @@ __global__ void __launch_bounds__(CUBE_THREADS) unpack_kernel(const void *cube, 
 }
 
 // Zeroes the entries whose count is not 0 (every other entry is zero
-// already), and the counters: the counts are read, 52 bytes of a touched
-// entry are written (mixed).  Against setting the whole cube to zero at the HBM peak: 6.7e7
-// entries, 31 % touched, 518 -> 221 us; 2.7e8 entries, 2.6 % touched, 2053 ->
-// 245 us.  A cube touched throughout would cost 4 bytes in 52 more.
-__global__ void __launch_bounds__(CUBE_THREADS) zero_kernel(void *cube, double *master, uint32_t *count,
+// already), and the counters: the counts are read, 20 bytes of a touched entry
+// are written (mixed), and its master's 32 where its moved bit is set.  Against
+// setting the whole cube to zero at the HBM peak: 6.7e7 entries, 31 % touched,
+// 518 -> 221 -> 146 us (with every touched entry's master, with the moved ones
+// only); 1.3e8 entries, 15 % touched, 1029 -> 268 -> 189 us; 2.7e8 entries, 2.6 %
+// touched, 2053 -> 245 -> 237 us (eight entries a thread: the counts' latency;
+// four 300).  A cube touched and moved throughout would cost 4 bytes in 52 more.
+__global__ void __launch_bounds__(CUBE_THREADS) zero_kernel(void *cube, double *master, uint32_t *moved, uint32_t *count,
                                                             DevStats *stats, int fp64, int64_t n)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) *stats = DevStats{};
-    for (int64_t b = (int64_t)blockIdx.x * CUBE_TILE + threadIdx.x; b < n; b += (int64_t)gridDim.x * CUBE_TILE) {
-        uint32_t c[CUBE_UNROLL];
+    for (int64_t b0 = (int64_t)blockIdx.x * ZERO_TILE; b0 < n; b0 += (int64_t)gridDim.x * ZERO_TILE) {
+        const int64_t b = b0 + threadIdx.x;
+        uint32_t c[ZERO_UNROLL];
 #pragma unroll
-        for (int q = 0; q < CUBE_UNROLL; ++q) {
+        for (int q = 0; q < ZERO_UNROLL; ++q) {
             const int64_t i = b + q * CUBE_THREADS;
             c[q] = i < n ? count[i] : 0u;
         }
+        const uint32_t word = moved_word<ZERO_UNROLL>(moved, b, n);
+        if (word != 0u) moved[moved_at(b)] = 0u;   // (its own lane's)
 #pragma unroll
-        for (int q = 0; q < CUBE_UNROLL; ++q) {
+        for (int q = 0; q < ZERO_UNROLL; ++q) {
             const int64_t i = b + q * CUBE_THREADS;
+            const uint32_t mv = __shfl_sync(0xffffffffu, word, q);
             if (c[q] == 0u) continue;
             if (fp64)
                 store_zero32(reinterpret_cast<double *>(cube) + 4 * i);
             else
                 reinterpret_cast<float4 *>(cube)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (master) store_zero32(master + 4 * i);
+            if (is_moved(mv, i)) store_zero32(master + 4 * i);
             count[i] = 0u;
         }
     }
@@ -282,7 +308,8 @@ __global__ void __launch_bounds__(SCAN_THREADS) sparse_scan_kernel(const uint32_
 }
 
 __global__ void __launch_bounds__(SPARSE_THREADS) sparse_write_kernel(const void *cube, const double *master,
-                                                                      const uint32_t *count, int fp64, int64_t n,
+                                                                      const uint32_t *moved, const uint32_t *count,
+                                                                      int fp64, int64_t n,
                                                                       const int64_t *tile_off, int64_t cap,
                                                                       int64_t *idx_out, float *sum_wv, float *sum_w,
                                                                       float *sum_wvv, uint32_t *cnt_out)
@@ -306,7 +333,7 @@ __global__ void __launch_bounds__(SPARSE_THREADS) sparse_write_kernel(const void
             const int64_t q = pos + before + __popc(bal & ((1u << lane) - 1u));
             if (q < cap) {
                 float e[4];
-                entry_value(load_entry(cube, master, fp64, i), fp64, e);
+                entry_value(load_entry(cube, master, moved && is_moved(moved[i >> 5], i), fp64, i), fp64, e);
                 idx_out[q] = i;
                 if (sum_wv) {
                     sum_wv[2 * q] = e[0];
@@ -330,11 +357,16 @@ __global__ void __launch_bounds__(SPARSE_THREADS) sparse_write_kernel(const void
 // entry and cleared (the exact widening of each component), so the FP32
 // partials start again from zero.  Nothing else touches the cube meanwhile
 // (the handle's stream orders it after the run's stacking).
-__global__ void fold_kernel(float4 *cube, double *master, int64_t n)
+__global__ void fold_kernel(float4 *cube, double *master, uint32_t *moved, int64_t n)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 c = cube[i];
-        if (c.x != 0.f || c.y != 0.f || c.z != 0.f || c.w != 0.f) {
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t b = tid & ~(int64_t)31; b < n; b += (int64_t)gridDim.x * blockDim.x) {   // 32 entries, a word, a warp
+        const int64_t i = b + (tid & 31);
+        const float4 c = i < n ? cube[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool nonzero = c.x != 0.f || c.y != 0.f || c.z != 0.f || c.w != 0.f;
+        const unsigned bits = __ballot_sync(0xffffffffu, nonzero);
+        if (bits != 0u && (tid & 31) == 0) moved[b >> 5] |= bits;
+        if (nonzero) {
             double *m = master + 4 * i;
             m[0] += (double)c.x;
             m[1] += (double)c.y;
@@ -345,43 +377,43 @@ __global__ void fold_kernel(float4 *cube, double *master, int64_t n)
     }
 }
 
-cudaError_t launch_fold(void *cube, double *master, int64_t n, cudaStream_t st)
+cudaError_t launch_fold(void *cube, double *master, uint32_t *moved, int64_t n, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
     int64_t blocks = (n + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    fold_kernel<<<(unsigned)blocks, 256, 0, st>>>(reinterpret_cast<float4 *>(cube), master, n);
+    fold_kernel<<<(unsigned)blocks, 256, 0, st>>>(reinterpret_cast<float4 *>(cube), master, moved, n);
     return cudaGetLastError();
 }
 
-static unsigned cube_blocks(int64_t n)
+static unsigned cube_blocks(int64_t n, int tile = CUBE_TILE)
 {
-    const int64_t tiles = (n + CUBE_TILE - 1) / CUBE_TILE;
+    const int64_t tiles = (n + tile - 1) / tile;
     return (unsigned)(tiles < 152 * 16 ? tiles : 152 * 16);
 }
 
-cudaError_t launch_unpack(const void *cube, const double *master, const uint32_t *count, int fp64, int all, int64_t n,
-                          void *sum_wv, void *sum_w, void *sum_wvv, uint32_t *cnt_out, int out_f64, cudaStream_t st)
+cudaError_t launch_unpack(const void *cube, const double *master, const uint32_t *moved, const uint32_t *count, int fp64,
+                          int all, int64_t n, void *sum_wv, void *sum_w, void *sum_wvv, uint32_t *cnt_out, int out_f64, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
     // one store per (re, im) pair, or one per value when sum_wv starts off a pair's boundary
     const int pair = ((uintptr_t)sum_wv % (out_f64 ? 16 : 8)) == 0;
     if (out_f64)
-        unpack_kernel<double><<<cube_blocks(n), CUBE_THREADS, 0, st>>>(cube, master, count, fp64, all, pair, n,
+        unpack_kernel<double><<<cube_blocks(n), CUBE_THREADS, 0, st>>>(cube, master, moved, count, fp64, all, pair, n,
                                                                        (double *)sum_wv, (double *)sum_w,
                                                                        (double *)sum_wvv, cnt_out);
     else
-        unpack_kernel<float><<<cube_blocks(n), CUBE_THREADS, 0, st>>>(cube, master, count, fp64, all, pair, n,
+        unpack_kernel<float><<<cube_blocks(n), CUBE_THREADS, 0, st>>>(cube, master, moved, count, fp64, all, pair, n,
                                                                       (float *)sum_wv, (float *)sum_w,
                                                                       (float *)sum_wvv, cnt_out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_zero_touched(void *cube, double *master, uint32_t *count, DevStats *stats, int fp64, int64_t n,
-                                cudaStream_t st)
+cudaError_t launch_zero_touched(void *cube, double *master, uint32_t *moved, uint32_t *count, DevStats *stats, int fp64,
+                                int64_t n, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    zero_kernel<<<cube_blocks(n), CUBE_THREADS, 0, st>>>(cube, master, count, stats, fp64, n);
+    zero_kernel<<<cube_blocks(n, ZERO_TILE), CUBE_THREADS, 0, st>>>(cube, master, moved, count, stats, fp64, n);
     return cudaGetLastError();
 }
 
@@ -395,13 +427,14 @@ cudaError_t launch_sparse_count(const uint32_t *count, int64_t n, uint32_t *tile
     return cudaGetLastError();
 }
 
-cudaError_t launch_sparse_write(const void *cube, const double *master, const uint32_t *count, int fp64, int64_t n,
+cudaError_t launch_sparse_write(const void *cube, const double *master, const uint32_t *moved, const uint32_t *count,
+                                int fp64, int64_t n,
                                 const int64_t *tile_off, int64_t cap, int64_t *index, float *sum_wv, float *sum_w,
                                 float *sum_wvv, uint32_t *cnt_out, cudaStream_t st)
 {
     const int64_t ntile = sparse_tiles(n);
     if (ntile == 0 || cap == 0) return cudaSuccess;
-    sparse_write_kernel<<<(unsigned)ntile, SPARSE_THREADS, 0, st>>>(cube, master, count, fp64, n, tile_off, cap, index,
+    sparse_write_kernel<<<(unsigned)ntile, SPARSE_THREADS, 0, st>>>(cube, master, moved, count, fp64, n, tile_off, cap, index,
                                                                    sum_wv, sum_w, sum_wvv, cnt_out);
     return cudaGetLastError();
 }

@@ -276,6 +276,7 @@ extern "C" int vista_stack_noalloc(const vista_cube_desc *c, const vista_source_
     a.g = CubeGeom{c->nu, c->nv, c->nrest, c->npol, gu, gv, c->hermitian_fold, 0};
     a.cube = cube4;
     a.cube_master = nullptr;
+    a.moved = nullptr;
     a.comp = 0;   // the caller's cube: plain float4 sums
     a.count = count;
     a.stats = (DevStats *)(b + o_stats);

@@ -344,7 +344,7 @@ static cudaError_t after_run(vista_stack *h, uint64_t nvis)
     if (h->nvis_since_fold < FOLD_DEPTH * (uint64_t)h->nentries) return cudaSuccess;
     h->nvis_since_fold = 0;
     if (h->timing) h->tacc.launches += 1;
-    return launch_fold(h->cube, h->cube_master, h->nentries, h->stream);
+    return launch_fold(h->cube, h->cube_master, h->moved, h->nentries, h->stream);
 }
 
 extern "C" int vista_run(vista_stack *h)
@@ -722,6 +722,7 @@ extern "C" int vista_run(vista_stack *h)
         a.g = g;
         a.cube = h->cube;
         a.cube_master = h->cube_master;
+        a.moved = h->moved;
         a.comp = h->cube_master ? 1 : 0;
         a.count = h->count;
         a.stats = h->stats;

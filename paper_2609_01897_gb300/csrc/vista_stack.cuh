@@ -224,6 +224,8 @@ __global__ void __launch_bounds__(KMAX_THREADS, (min_blocks<P>())) stack_mixed(R
             atomicAdd(ck_dst + 1, widen(ck_took.y));
             atomicAdd(ck_dst + 2, widen(ck_took.z));
             atomicAdd(ck_dst + 3, widen(ck_took.w));
+            const int64_t ce = (ck_dst - a.cube_master) >> 2;
+            atomicOr(a.moved + (ce >> 5), 1u << (ce & 31));
             n_red += 4;
             ck_dst = nullptr;
         }
