@@ -296,10 +296,10 @@ __device__ __forceinline__ float2 subtract_fit(const EntryFF &v, float2 x, const
 // the touched ones lie together, and their warps, bound by latency, then run
 // beside others that stream.  2.7e8 entries of four planes, 10 % of the cells
 // and 6.3 % of the entries touched, order 1: 3704 us when every entry was read
-// twice, 1125 us in cell order with the counts a word at a time, 963 us so
-// (5.1 TB/s of the 4.9 GB moved; the second pass finds its entries evicted from
-// L2).  Slower: several warps a cell (1500 us: their FP64 reductions and
-// solves), entries of two or four rows loaded together (1780, 2460: registers).
+// twice, 1125 us in cell order with the counts a word at a time, 956 us so (the
+// second pass finds its entries evicted from L2).  Slower: several warps a cell
+// (1500 us: their FP64 reductions and solves), entries of two or four rows loaded
+// together (1780, 2460: registers).
 constexpr int CELL_UNROLL = 8, WIDE_LOADS = 8, CELL_THREADS = 128;
 
 // Bit q: entry base + 32 q + lane of the cell is touched.
