@@ -10,13 +10,30 @@ namespace vista {
 
 // ---------------------------------------------------------------- helpers
 
-// Largest s with off[s] <= x (off non-decreasing, off[0] = 0).
+// Largest s with off[s] <= x (off non-decreasing, off[0] = 0).  The table is
+// read through the read-only path: nothing may write it while the kernel is on
+// the chip (a table uploaded before the pre-pass, not one that the pre-pass forms).
 __device__ __forceinline__ int find_owner(const int64_t *__restrict__ off, int n, int64_t x)
 {
     int lo = 0, hi = n - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
         if (__ldg(off + mid) <= x)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    return lo;
+}
+
+// The same over a table that an earlier kernel of the chain writes: ordinary
+// loads (see chain_begin).
+__device__ __forceinline__ int find_owner_chained(const int64_t *off, int n, int64_t x)
+{
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        int mid = (lo + hi + 1) >> 1;
+        if (off[mid] <= x)
             lo = mid;
         else
             hi = mid - 1;
@@ -35,6 +52,12 @@ __device__ __forceinline__ int find_owner(const int64_t *__restrict__ off, int n
 // single wait.  The stacking kernels are launched as usual: their persistent
 // blocks, waiting on the chip before the pre-pass has ended, cost the FP64
 // form 6 % and an archive stack 1 %.
+//
+// A chained kernel's blocks are on the chip while the kernel before them still
+// writes.  What the chain writes is therefore never read through the read-only
+// path (__ldg, find_owner): such loads are only defined for data that nothing
+// writes during the whole life of the kernel, waiting part included, and may
+// be moved across the wait.
 
 __device__ __forceinline__ void chain_begin()
 {

@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(256) k_items(RunArgs a)
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nb = (int64_t)a.nsrc * so.nstripe;
     if (p >= so.ioff[nb] || p >= so.max_items) return;
-    const int i = find_owner(so.ioff, (int)nb, p);
+    const int i = find_owner_chained(so.ioff, (int)nb, p);
     const int R = so.rows_per_item;
     const Bucket bk = bucket_at(a, i);
     const int st = bk.s, w = bk.w;
