@@ -529,13 +529,15 @@ __global__ void __launch_bounds__(KMAX_THREADS, (min_blocks<P>())) stack_mixed(R
             // one float4 reduction per (cell, rest bin, pol) and the counts.
             //
             // With checkpoints (comp), in one drain in CKPT_EVERY (drawn by the
-            // warp's sequence) the writing lanes also move one entry each (their
-            // first bin, a pol that differs from lane to lane and drain to drain)
-            // into the FP64 master cube: 16-byte atomic exchange with zero, and
-            // the FP64 reductions of the value taken at the lane's next exchange
-            // (or at the end), so nothing waits on a returned value.  An entry's
-            // FP32 sum thus holds only the additions since its last checkpoint,
-            // about CKPT_EVERY x P of them.
+            // warp's sequence) the writing lanes also move one entry each into the
+            // FP64 master cube: 16-byte atomic exchange with zero, and the FP64
+            // reductions of the value taken at the lane's next exchange (or at the
+            // end), so nothing waits on a returned value.  The entry is one of
+            // those the lane has just added to, its bin and pol drawn anew each
+            // time (a bin may be no channel's first: the upper half of a channel
+            // two bins wide, a window's last bin), so that every entry's FP32 sum
+            // holds only the additions since its last checkpoint, about
+            // CKPT_EVERY x P x (bins a lane writes) of them.
             auto drain = [&]() {
                 __syncwarp();
                 const uint32_t k = count < 32u ? count : 32u;
@@ -641,18 +643,19 @@ __global__ void __launch_bounds__(KMAX_THREADS, (min_blocks<P>())) stack_mixed(R
                     };
                     if (emit) add(e, z, zn);
                     if (emit2) add(e + npol_c, y, rn);
-                    if (service && emit) {
+                    if (service && (emit || emit2)) {
                         // complete the lane's previous exchange, whose value has long
                         // arrived, then take the chosen entry's FP32 sums
                         flush_ckpt();
-                        const int64_t ce = e + ((rnd >> 20) + (uint32_t)lane) % P;
+                        const bool second = emit2 && (!emit || (rnd >> 28 & 1u));
+                        const int64_t ce = e + (second ? npol_c : 0) + ((rnd >> 20) + (uint32_t)lane) % P;
                         ck_took = atomicExch(cube4 + ce, make_float4(0.f, 0.f, 0.f, 0.f));
                         ck_dst = a.cube_master + 4 * ce;
                         ++n_red;
                     }
                 } else if (on) {
                     const int64_t kt = chf0 + k0 + src;   // the run's channel-table entry
-                    const int rb = a.chf[kt].nb;
+                    const int rb = a.chf[kt].nb, ck_b = (int)((rnd >> 24) % (uint32_t)rb);   // (a staged run's channel has a bin)
                     for (int b = 0; b < rb; ++b) {
                         const float ww = b == 0 ? r0 : b == 1 ? r1 : far_bin_weight(a.chd + kt, b);
                         const int64_t e2 = (int64_t)rc * cell_entries + (int64_t)(rj + b) * npol_c;
@@ -662,7 +665,7 @@ __global__ void __launch_bounds__(KMAX_THREADS, (min_blocks<P>())) stack_mixed(R
                             red_add4(cube4 + e2 + plane[p], ww * v[p][0], ww * v[p][1], ww * v[p][2], ww * v[p][3]);
                             atomicAdd(a.count + e2 + plane[p], rn[p]);
                             n_red += 2;
-                            if (service && b == 0 && p == (int)(((rnd >> 20) + (uint32_t)lane) % P)) {
+                            if (service && b == ck_b && p == (int)(((rnd >> 20) + (uint32_t)lane) % P)) {
                                 flush_ckpt();
                                 ck_took = atomicExch(cube4 + e2 + plane[p], make_float4(0.f, 0.f, 0.f, 0.f));
                                 ck_dst = a.cube_master + 4 * (e2 + plane[p]);
