@@ -124,13 +124,14 @@ static __device__ __noinline__ float far_bin_weight(const ChanD *cd, int b) { re
 
 // A float as a double, exactly, by moving its IEEE-754 fields (integer
 // instructions; the FP64 unit converts slowly).  Zero and subnormal inputs
-// give zero (below 1.2e-38), infinities and NaNs do not occur in the sums.
+// give zero (below 1.2e-38); infinities and NaNs stay what they are.
 __device__ __forceinline__ double widen(float x)
 {
     const uint32_t b = __float_as_uint(x);
     const uint32_t e = (b >> 23) & 0xffu;
     if (e == 0u) return 0.0;
-    const uint32_t hi = (b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3);
+    const uint32_t e64 = e == 0xffu ? 0x7ffu : e + 896u;
+    const uint32_t hi = (b & 0x80000000u) | (e64 << 20) | ((b & 0x7fffffu) >> 3);
     return __hiloint2double((int)hi, (int)(b << 29));
 }
 
