@@ -1,8 +1,8 @@
 // Device helpers for kernels that walk the cube's entries (readback, zeroing,
-// continuum subtraction): float-pair arithmetic that stays off the FP64 pipe
-// (about two lanes a clock and SM on GB300: widening, adding and narrowing the
-// four sums of every entry of a 6.7e7-entry cube took 1.3 ms there, three
-// times its memory time), and 32-byte accesses.
+// continuum subtraction): conversions and float-pair arithmetic that stay off the
+// FP64 pipe (about two lanes a clock and SM on GB300: widening, adding and
+// narrowing the four sums of every entry of a 6.7e7-entry cube took 1.3 ms there,
+// three times its memory time), and 32-byte accesses.
 #pragma once
 #include <cstdint>
 
@@ -61,20 +61,32 @@ __device__ __forceinline__ float2 add_ff(float2 a, float b)   // (a.x + a.y) + b
     return make_float2(hi, lo - (hi - t));
 }
 
-static __device__ __noinline__ float sum_f32_slow(float c, double m) { return (float)((double)c + m); }
-
-// fl32(c + m) of an entry's FP32 partial and FP64 master sum (within 2^-40 of
-// a unit in the last place of the rounded FP64 sum).  Masters outside the
-// normal floats' range (infinities and NaNs among them) take the FP64 form.
-__device__ __forceinline__ float sum_f32(float c, double m)
+// A float as a double and a double rounded to a float (to nearest, ties to even),
+// by moving the fields: integer instructions, where the FP64 unit's conversions
+// are as slow as its additions.
+static __device__ __noinline__ double widen_slow(float x) { return (double)x; }    // subnormal, infinite, NaN
+static __device__ __noinline__ float narrow_slow(double x) { return (float)x; }    // outside the normal floats
+__device__ __forceinline__ double widen_exact(float x)
 {
-    const int e = (__double2hiint(m) >> 20) & 0x7ff;
-    if (e == 0) return c;   // zero, or below 2^-1022
-    if (__builtin_expect(e < 897 || e > 1150, 0)) return sum_f32_slow(c, m);
-    const float2 s = split_double(m);
-    const float t = s.x + c;
-    if (!(fabsf(t) < __int_as_float(0x7f800000))) return t;   // c infinite or NaN, or an overflow
-    return add_ff(s, c).x;
+    const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+    if (__builtin_expect(e - 1u >= 254u && (b << 1) != 0u, 0)) return widen_slow(x);
+    return __hiloint2double((int)((b & 0x80000000u) | (e ? ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3) : 0u)), (int)(b << 29));
+}
+__device__ __forceinline__ float narrow(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffull;
+    if (__builtin_expect((uint32_t)(m >> 52) - 897u > 253u, 0)) return narrow_slow(x);
+    const uint32_t f = (uint32_t)((m + 0x0fffffffull + ((m >> 29) & 1ull)) >> 29) - (896u << 23);   // (may round up to infinity)
+    return __uint_as_float(f | ((uint32_t)(b >> 32) & 0x80000000u));
+}
+
+// An entry's FP32 partials c and FP64 master sums m, added in FP64 and rounded
+// to floats.  Four FP64 operations: only entries with a master pay them (one
+// touched entry in eight as a rule), beside the memory's time.
+__device__ __forceinline__ float4 sum_f32(float4 c, const Double4 &m)
+{
+    return make_float4(narrow(widen_exact(c.x) + m.x), narrow(widen_exact(c.y) + m.y), narrow(widen_exact(c.z) + m.z),
+                       narrow(widen_exact(c.w) + m.w));
 }
 
 }  // namespace vista

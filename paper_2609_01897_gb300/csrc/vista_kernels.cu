@@ -104,10 +104,11 @@ __global__ void __launch_bounds__(128) debug_fp64(RunArgs a, int src, double *ph
 struct RawEntry {
     float4 f;
     Double4 d;
+    bool has_master;
 };
 __device__ __forceinline__ RawEntry load_entry(const void *cube, const double *master, bool has_master, int fp64, int64_t i)
 {
-    RawEntry r{make_float4(0.f, 0.f, 0.f, 0.f), Double4{0.0, 0.0, 0.0, 0.0}};
+    RawEntry r{make_float4(0.f, 0.f, 0.f, 0.f), Double4{0.0, 0.0, 0.0, 0.0}, has_master};
     if (!fp64) r.f = reinterpret_cast<const float4 *>(cube)[i];
     if (fp64) r.d = load_double4(reinterpret_cast<const double *>(cube) + 4 * i);
     else if (has_master) r.d = load_double4(master + 4 * i);
@@ -123,10 +124,11 @@ __device__ __forceinline__ void entry_value(const RawEntry &r, int fp64, T (&e)[
             e[2] = (float)r.d.z;
             e[3] = (float)r.d.w;
         } else {
-            e[0] = sum_f32(r.f.x, r.d.x);
-            e[1] = sum_f32(r.f.y, r.d.y);
-            e[2] = sum_f32(r.f.z, r.d.z);
-            e[3] = sum_f32(r.f.w, r.d.w);
+            const float4 q = r.has_master ? sum_f32(r.f, r.d) : r.f;
+            e[0] = q.x;
+            e[1] = q.y;
+            e[2] = q.z;
+            e[3] = q.w;
         }
     } else {
         e[0] = fp64 ? r.d.x : (double)r.f.x + r.d.x;
