@@ -101,42 +101,52 @@ __global__ void __launch_bounds__(128) debug_fp64(RunArgs a, int src, double *ph
 // Entry i's four sums (re and im of sum wV, sum w, sum w|V|^2): the FP64
 // cube, or the mixed cube's float4 sums since the last checkpoint plus its
 // FP64 master sums, as doubles or rounded to floats.
+template <bool FP64>
 struct RawEntry {
     float4 f;
     Double4 d;
     bool has_master;
-};
-__device__ __forceinline__ RawEntry load_entry(const void *cube, const double *master, bool has_master, int fp64, int64_t i)
-{
-    RawEntry r{make_float4(0.f, 0.f, 0.f, 0.f), Double4{0.0, 0.0, 0.0, 0.0}, has_master};
-    if (!fp64) r.f = reinterpret_cast<const float4 *>(cube)[i];
-    if (fp64) r.d = load_double4(reinterpret_cast<const double *>(cube) + 4 * i);
-    else if (has_master) r.d = load_double4(master + 4 * i);
-    return r;
-}
-template <typename T>
-__device__ __forceinline__ void entry_value(const RawEntry &r, int fp64, T (&e)[4])
-{
-    if constexpr (sizeof(T) == 4) {
-        if (fp64) {
-            e[0] = (float)r.d.x;
-            e[1] = (float)r.d.y;
-            e[2] = (float)r.d.z;
-            e[3] = (float)r.d.w;
+    __device__ __forceinline__ void load(const void *cube, const double *master, bool has, int64_t i)
+    {
+        if constexpr (FP64) {
+            d = load_double4(reinterpret_cast<const double *>(cube) + 4 * i);
         } else {
-            const float4 q = r.has_master ? sum_f32(r.f, r.d) : r.f;
+            f = reinterpret_cast<const float4 *>(cube)[i];
+            has_master = has;
+            if (has) d = load_double4(master + 4 * i);
+        }
+    }
+    __device__ __forceinline__ void value(float (&e)[4]) const
+    {
+        if constexpr (FP64) {
+            e[0] = narrow(d.x);
+            e[1] = narrow(d.y);
+            e[2] = narrow(d.z);
+            e[3] = narrow(d.w);
+        } else {
+            const float4 q = has_master ? sum_f32(f, d) : f;
             e[0] = q.x;
             e[1] = q.y;
             e[2] = q.z;
             e[3] = q.w;
         }
-    } else {
-        e[0] = fp64 ? r.d.x : (double)r.f.x + r.d.x;
-        e[1] = fp64 ? r.d.y : (double)r.f.y + r.d.y;
-        e[2] = fp64 ? r.d.z : (double)r.f.z + r.d.z;
-        e[3] = fp64 ? r.d.w : (double)r.f.w + r.d.w;
     }
-}
+    __device__ __forceinline__ void value(double (&e)[4]) const
+    {
+        if constexpr (FP64) {
+            e[0] = d.x;
+            e[1] = d.y;
+            e[2] = d.z;
+            e[3] = d.w;
+        } else {
+            const Double4 m = has_master ? d : Double4{0.0, 0.0, 0.0, 0.0};
+            e[0] = widen_exact(f.x) + m.x;
+            e[1] = widen_exact(f.y) + m.y;
+            e[2] = widen_exact(f.z) + m.z;
+            e[3] = widen_exact(f.w) + m.w;
+        }
+    }
+};
 
 // The cube -> caller arrays.  An entry whose count is 0 has had no
 // contribution, so only its count is read and zeros are written: 24 bytes an
@@ -147,10 +157,17 @@ __device__ __forceinline__ void entry_value(const RawEntry &r, int fp64, T (&e)[
 // block apart, so that every access of a warp is contiguous and the counts of
 // all of them are in flight together.  Before (every entry read, widened,
 // added and narrowed on the FP64 pipe, which bound it) and now: 6.7e7 entries,
-// 31 % touched, 1478 -> 443 us (468 with the masters that are zero read too);
-// 2.7e8 entries, 2.6 % touched, 5902 -> 1365 us; 4.2e6 entries, 10 % touched, 96
+// 31 % touched, 1478 -> 403 us (468 with the masters that are zero read too);
+// 2.7e8 entries, 2.6 % touched, 5902 -> 1392 us; 4.2e6 entries, 10 % touched, 96
 // -> 23 us.  It is at the rate of its writes: streaming stores, 16-byte stores of
-// four entries a thread and eight entries a thread were level or slower.
+// four entries a thread and eight entries a thread were level or slower.  Sums
+// are read only where some array of sums is asked for.  The FP64 cube has a form
+// of its own: without the float sums and the moved bits it needs 64 registers
+// instead of 80, and the next tile's counts are loaded under this tile's sums, which
+// a call for one array, with few writes to wait for, would otherwise wait for (1.7e7
+// entries of four planes, sum_w alone 138 -> 72 us, the counts alone 138 -> 29;
+// all arrays 146 -> 110).  On the mixed cube the early counts cost registers
+// (1392 -> 1747 us on the 2.7e8 entries).
 constexpr int CUBE_THREADS = 256, CUBE_UNROLL = 4, CUBE_TILE = CUBE_THREADS * CUBE_UNROLL;
 constexpr int ZERO_UNROLL = 8, ZERO_TILE = CUBE_THREADS * ZERO_UNROLL;
 
@@ -168,37 +185,50 @@ __device__ __forceinline__ uint32_t moved_word(const uint32_t *moved, int64_t b,
     return moved && (threadIdx.x & 31) < N && 32 * w < n ? moved[w] : 0u;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(CUBE_THREADS) unpack_kernel(const void *cube, const double *master,
-                                                              const uint32_t *moved, const uint32_t *count, int fp64, int all, int pair,
-                                                              int64_t n, T *sum_wv, T *sum_w, T *sum_wvv,
-                                                              uint32_t *cnt_out)
+template <typename T, bool FP64>
+__global__ void __launch_bounds__(CUBE_THREADS, FP64 ? 4 : 3) unpack_kernel(const void *cube, const double *master,
+                                                                            const uint32_t *moved, const uint32_t *count,
+                                                                            int all, int pair, int64_t n, T *sum_wv,
+                                                                            T *sum_w, T *sum_wvv, uint32_t *cnt_out)
 {
     struct alignas(2 * sizeof(T)) Pair {
         T re, im;
     };
-    for (int64_t b0 = (int64_t)blockIdx.x * CUBE_TILE; b0 < n; b0 += (int64_t)gridDim.x * CUBE_TILE) {
-        const int64_t b = b0 + threadIdx.x;
-        uint32_t c[CUBE_UNROLL];
-        RawEntry r[CUBE_UNROLL];
+    const bool sums = sum_wv || sum_w || sum_wvv;   // (the counts alone: no entry is read)
+    const int64_t step = (int64_t)gridDim.x * CUBE_TILE;
+    uint32_t next[CUBE_UNROLL];
+    auto load_counts = [&](int64_t b, uint32_t (&c)[CUBE_UNROLL]) {
 #pragma unroll
         for (int q = 0; q < CUBE_UNROLL; ++q) {
             const int64_t i = b + q * CUBE_THREADS;
             c[q] = i < n ? count[i] : 0u;
         }
-        const uint32_t word = moved_word<CUBE_UNROLL>(moved, b, n);
+    };
+    if constexpr (FP64) load_counts((int64_t)blockIdx.x * CUBE_TILE + threadIdx.x, next);
+    for (int64_t b0 = (int64_t)blockIdx.x * CUBE_TILE; b0 < n; b0 += step) {
+        const int64_t b = b0 + threadIdx.x;
+        uint32_t c[CUBE_UNROLL], word = 0u;
+        RawEntry<FP64> r[CUBE_UNROLL];
+        if constexpr (FP64) {
+#pragma unroll
+            for (int q = 0; q < CUBE_UNROLL; ++q) c[q] = next[q];
+            if (b0 + step < n) load_counts(b + step, next);
+        } else {
+            load_counts(b, c);
+            if (sums) word = moved_word<CUBE_UNROLL>(moved, b, n);
+        }
 #pragma unroll
         for (int q = 0; q < CUBE_UNROLL; ++q) {
             const int64_t i = b + q * CUBE_THREADS;
-            const uint32_t mv = __shfl_sync(0xffffffffu, word, q);
-            if (i < n && (all || c[q] != 0u)) r[q] = load_entry(cube, master, is_moved(mv, i), fp64, i);
+            const uint32_t mv = FP64 ? 0u : __shfl_sync(0xffffffffu, word, q);
+            if (sums && i < n && (all || c[q] != 0u)) r[q].load(cube, master, is_moved(mv, i), i);
         }
 #pragma unroll
         for (int q = 0; q < CUBE_UNROLL; ++q) {
             const int64_t i = b + q * CUBE_THREADS;
             if (i >= n) break;
             T e[4] = {0, 0, 0, 0};
-            if (all || c[q] != 0u) entry_value(r[q], fp64, e);
+            if (sums && (all || c[q] != 0u)) r[q].value(e);
             if (sum_wv && pair) {
                 reinterpret_cast<Pair *>(sum_wv)[i] = Pair{e[0], e[1]};
             } else if (sum_wv) {
@@ -335,7 +365,15 @@ __global__ void __launch_bounds__(SPARSE_THREADS) sparse_write_kernel(const void
             const int64_t q = pos + before + __popc(bal & ((1u << lane) - 1u));
             if (q < cap) {
                 float e[4];
-                entry_value(load_entry(cube, master, moved && is_moved(moved[i >> 5], i), fp64, i), fp64, e);
+                if (fp64) {
+                    RawEntry<true> r;
+                    r.load(cube, nullptr, false, i);
+                    r.value(e);
+                } else {
+                    RawEntry<false> r;
+                    r.load(cube, master, moved && is_moved(moved[i >> 5], i), i);
+                    r.value(e);
+                }
                 idx_out[q] = i;
                 if (sum_wv) {
                     sum_wv[2 * q] = e[0];
@@ -400,14 +438,15 @@ cudaError_t launch_unpack(const void *cube, const double *master, const uint32_t
     if (n == 0) return cudaSuccess;
     // one store per (re, im) pair, or one per value when sum_wv starts off a pair's boundary
     const int pair = ((uintptr_t)sum_wv % (out_f64 ? 16 : 8)) == 0;
+    auto launch = [&](auto *kern, auto *wv, auto *w, auto *wvv) {
+        kern<<<cube_blocks(n), CUBE_THREADS, 0, st>>>(cube, master, moved, count, all, pair, n, wv, w, wvv, cnt_out);
+    };
     if (out_f64)
-        unpack_kernel<double><<<cube_blocks(n), CUBE_THREADS, 0, st>>>(cube, master, moved, count, fp64, all, pair, n,
-                                                                       (double *)sum_wv, (double *)sum_w,
-                                                                       (double *)sum_wvv, cnt_out);
+        launch(fp64 ? unpack_kernel<double, true> : unpack_kernel<double, false>, (double *)sum_wv, (double *)sum_w,
+               (double *)sum_wvv);
     else
-        unpack_kernel<float><<<cube_blocks(n), CUBE_THREADS, 0, st>>>(cube, master, moved, count, fp64, all, pair, n,
-                                                                      (float *)sum_wv, (float *)sum_w,
-                                                                      (float *)sum_wvv, cnt_out);
+        launch(fp64 ? unpack_kernel<float, true> : unpack_kernel<float, false>, (float *)sum_wv, (float *)sum_w,
+               (float *)sum_wvv);
     return cudaGetLastError();
 }
 
