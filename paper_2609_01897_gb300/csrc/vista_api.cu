@@ -25,21 +25,6 @@ bool is_fin(double x) { return std::isfinite(x); }
         if (!handle_live(h)) return fail(nullptr, VISTA_E_STATE, "unknown or closed handle"); \
     } while (0)
 
-// Row-ordering stripes: a few iv rows of the cube whose FP32 entries fit in
-// about 40 MB, so the cube region a stripe's work touches stays in L2; the
-// cell key inside a stripe must fit the shared-memory histogram.
-int stripe_geometry(vista_stack *h)
-{
-    const vista_cube_desc &d = h->desc;
-    int S = 1, nst = 1, ushift = 0, nuk = 1;
-    if (!stripe_layout(d.nu, d.nv, d.nrest, d.npol, MIN_STRIPES, &S, &nst, &ushift, &nuk)) return VISTA_E_RANGE;
-    h->stripe_rows = S;
-    h->nstripe = nst;
-    h->ushift = ushift;
-    h->nuk = nuk;
-    return VISTA_OK;
-}
-
 }  // namespace
 
 namespace vista {
@@ -211,7 +196,8 @@ extern "C" int vista_open_stack(const vista_cube_desc *d, vista_stack **out)
         h->f0 = d->rest_f0;
         h->df = d->rest_df;
     }
-    if (stripe_geometry(h) != VISTA_OK) {
+    int S, nst, ushift, nuk;
+    if (!stripe_layout(d->nu, d->nv, d->nrest, d->npol, 1, &S, &nst, &ushift, &nuk)) {
         delete h;
         return fail(nullptr, VISTA_E_RANGE, "cube too tall for the row ordering");
     }

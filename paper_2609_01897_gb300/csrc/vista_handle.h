@@ -140,8 +140,6 @@ struct vista_stack {
     cudaEvent_t xfer_ev[5] = {};
     cudaGraphExec_t gexec = nullptr;
     uint64_t graph_launches = 0;
-    // stripe geometry of the row ordering (depends on the cube only)
-    int32_t stripe_rows = 1, nstripe = 1, ushift = 0, nuk = 1;
     std::string msg;
     bool timing = false;
     std::vector<vista::Span> spans;

@@ -20,13 +20,23 @@ constexpr int MAX_STRIPES = 4096;         // stripes of the cube (shared-memory 
 // call holds the counts of 2048-row segments.
 constexpr int SEG_ROWS = 2048, SEG_ROWS_SMALL = 512;
 inline int segment_rows(int64_t rows) { return rows / SEG_ROWS < 2 * 152 ? SEG_ROWS_SMALL : SEG_ROWS; }
-// Stripes a handle's cube is cut into at the least (where it has the rows): a
-// block sorts one (window, stripe) bucket, so that a small cube, whose
-// entries would all fit one stripe, still spreads a window's sort over many
-// blocks (k_bucket_sort of one window of 10 001 rows 31 -> 7 us, of four of
-// 18 000 rows 68 -> 10 us; more, smaller items also fill the chip better when
-// a stack is small).
-constexpr int MIN_STRIPES = 32;
+// Stripes a run cuts the cube into at the least (where it has the rows): a block
+// sorts one (window, stripe) bucket, so that a small cube, whose entries would
+// all fit one stripe, still spreads a window's sort over many blocks (k_bucket_sort
+// of one window of 10 001 rows 31 -> 7 us, of four of 18 000 rows 68 -> 10 us;
+// more, smaller items also fill the chip better when a stack is small).  Many
+// windows are spread as they are, and each bucket costs a block, so the buckets
+// stay near eight a SM, but for those of more than 2048 keys, whose tables then
+// cost more than another block.  600 windows of 100 rows, pre-pass + stacking
+// kernel: into a 32 x 32 cube 125 + 62 us with 32 stripes, 58 + 57 with these two;
+// 64 x 64, 130 + 85 and 78 + 84; 256 x 256, 348 + 108 with two (16, as many
+// as the keys allow), 330 + 119 with these 32.  2000 windows into 32 x 32: 345 + 153
+// and 114 + 128; 100 windows are level.
+inline int min_stripes(int64_t windows, int64_t cells)
+{
+    const int64_t few = 8 * 152 / (windows > 0 ? windows : 1), big = cells / 2048, s = few > big ? few : big;
+    return s < 1 ? 1 : (s > 32 ? 32 : (int)s);
+}
 
 // Row-ordering stripes of a cube: S iv rows per stripe (sized so that a
 // stripe's cube entries, ~20 B each, stay near 40 MB and resident in L2, and

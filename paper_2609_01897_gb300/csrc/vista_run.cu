@@ -540,7 +540,6 @@ extern "C" int vista_run(vista_stack *h)
     std::vector<size_t> prep_src0, prep_off0;
     std::vector<SortLayout> layouts;
     size_t sort_bytes = 0;
-    const int nst = cfg.sort_rows ? h->nstripe : 1;
     int64_t rec_total = 0, cell_total = 0;
     uint64_t nvis_run = 0, bound_run = 0;
     std::vector<Copy2D> copies;
@@ -564,6 +563,13 @@ extern "C" int vista_run(vista_stack *h)
         int64_t max_items = 0, rows = 0;
         for (int i : windows) rows += h->pending[(size_t)i].d.nrow;
         const int seg = segment_rows(rows);
+        // row-ordering stripes: a few iv rows of the cube whose FP32 entries fit
+        // in about 40 MB, so the cube region a stripe's work touches stays in L2
+        int stripe_rows = c.nv, nst = 1, ushift = 0, nuk = 1;
+        if (cfg.sort_rows &&
+            !stripe_layout(c.nu, c.nv, c.nrest, c.npol, min_stripes((int64_t)m, (int64_t)c.nu * c.nv), &stripe_rows, &nst,
+                           &ushift, &nuk))
+            return fail(h, VISTA_E_RANGE, "cube too tall for the row ordering");   // (open has refused such cubes)
         for (size_t t = 0; t < m; ++t) {
             const int i = windows[t], cw = width[t];
             const SrcHost &s = h->pending[(size_t)i];
@@ -658,7 +664,7 @@ extern "C" int vista_run(vista_stack *h)
             }
             roff[t + 1] = roff[t] + d.nrow;
             soff[t + 1] = soff[t] + (d.nrow + seg - 1) / seg;
-            max_items += (int64_t)d.nchunk * ((d.nrow + cfg.rows_per_item - 1) / cfg.rows_per_item + h->nstripe);
+            max_items += (int64_t)d.nchunk * ((d.nrow + cfg.rows_per_item - 1) / cfg.rows_per_item + nst);
             d.guvw = d.uvw;
             if (s.has_rot) {
                 d.rot1 = (int32_t)(rots.size() / 9) + 1;
@@ -680,6 +686,10 @@ extern "C" int vista_run(vista_stack *h)
         pr.args.so.nseg_total = soff[m];
         pr.args.so.max_items = max_items;
         pr.args.so.nclass = (int32_t)(c1 - c0);
+        pr.args.so.stripe_rows = stripe_rows;
+        pr.args.so.nstripe = nst;
+        pr.args.so.ushift = ushift;
+        pr.args.so.nuk = nuk;
         preps.push_back(pr);
         layouts.push_back(sort_layout(roff[m], (int64_t)m * nst, max_items, soff[m], nst, c1 - c0));
         sort_bytes = std::max(sort_bytes, layouts.back().total);
@@ -741,10 +751,6 @@ extern "C" int vista_run(vista_stack *h)
         so.items = (Item *)(b + L.items);
         so.ctr = (uint32_t *)(b + L.ctr);
         so.sorted = cfg.sort_rows;
-        so.stripe_rows = cfg.sort_rows ? h->stripe_rows : c.nv;
-        so.nstripe = nst;
-        so.ushift = h->ushift;
-        so.nuk = h->nuk;
         so.rows_per_item = cfg.rows_per_item;
         for (size_t ci = preps[pi].c0; ci < preps[pi].c1; ++ci) {
             classes[ci].args = a;
