@@ -17,8 +17,8 @@
 // instruction and read the tables again for every row).  Bound by L1 lines a
 // load (wide windows, whose outputs' contributors lie several channels apart)
 // and by latency (narrow ones).  Kernel time, 12 000 rows x 3840 channels x 4
-// pols onto 1024: 437 -> 380 us (1.92 GB, 5.0 TB/s); 27 090 rows x 120
-// channels x 2 pols of FP16 onto 150: 87 -> 50 us.  Eight rows a tile: four
+// pols onto 1024: 437 -> 385 us (1.92 GB, 5.0 TB/s); 27 090 rows x 120
+// channels x 2 pols of FP16 onto 150: 87 -> 43 us.  Eight rows a tile: four
 // cost 6 % on the FP16 window, sixteen 10 % on the wide one; blocks of 128
 // columns 7 % on the wide one.  The tables were built on the host before
 // (130 and 50 us a call around the kernels, 65 and 40 us now).
@@ -205,20 +205,18 @@ __global__ void __launch_bounds__(COLS, 14) k_regrid(RegridArgs a)
 #pragma unroll
             for (int r = 0; r < R; ++r) fl[r] = 0u;
         }
-        float wc[RP], ws[RP];
+        float2 ph[RP];
 #pragma unroll
-        for (int i = 0; i < RP; ++i) {
-            const float2 ph = shift_phasor(tau[i].x, tau[i].y, nh, nl);
-            wc[i] = w * ph.x;
-            ws[i] = w * ph.y;
-        }
+        for (int i = 0; i < RP; ++i) ph[i] = shift_phasor(tau[i].x, tau[i].y, nh, nl);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const float c = P == 1 ? wc[r / P] : __shfl_sync(0xffffffffu, wc[r / P], r % P, P);
-            const float s = P == 1 ? ws[r / P] : __shfl_sync(0xffffffffu, ws[r / P], r % P, P);
+            const float c = P == 1 ? ph[r / P].x : __shfl_sync(0xffffffffu, ph[r / P].x, r % P, P);
+            const float s = P == 1 ? ph[r / P].y : __shfl_sync(0xffffffffu, ph[r / P].y, r % P, P);
             if (use && fl[r] == 0u) {
-                sr[r] = __fmaf_rn(v[r].x, c, __fmaf_rn(-v[r].y, s, sr[r]));
-                si[r] = __fmaf_rn(v[r].x, s, __fmaf_rn(v[r].y, c, si[r]));
+                // (weighting the phasors instead would save two operations of six and
+                // add a rounding: rms errors 5 to 20 % larger)
+                sr[r] = __fmaf_rn(w, __fmaf_rn(v[r].x, c, -__fmul_rn(v[r].y, s)), sr[r]);
+                si[r] = __fmaf_rn(w, __fmaf_rn(v[r].x, s, __fmul_rn(v[r].y, c)), si[r]);
                 sw[r] += w;
             }
         }
