@@ -17,11 +17,13 @@
 // instruction and read the tables again for every row).  Bound by L1 lines a
 // load (wide windows, whose outputs' contributors lie several channels apart)
 // and by latency (narrow ones).  Kernel time, 12 000 rows x 3840 channels x 4
-// pols onto 1024: 437 -> 385 us (1.92 GB, 5.0 TB/s); 27 090 rows x 120
-// channels x 2 pols of FP16 onto 150: 87 -> 43 us.  Eight rows a tile: four
-// cost 6 % on the FP16 window, sixteen 10 % on the wide one; blocks of 128
-// columns 7 % on the wide one.  The tables were built on the host before
-// (130 and 50 us a call around the kernels, 65 and 40 us now).
+// pols onto 1024: 437 -> 362 us (1.92 GB, 5.3 TB/s); 27 090 rows x 120
+// channels x 2 pols of FP16 onto 150: 87 -> 43 us.  Rows a tile by shape, see
+// launch_regrid_p: eight are 6 % better than four on the FP16 window and 5 % worse
+// on the wide one; blocks of 128 columns cost 7 % on the wide one.  Outputs of few
+// columns have a form of their own, k_regrid_pols.  The tables were built on the host
+// before (130 and 50 us a call around the kernels, 65 and 40 us now).
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <vector>
@@ -55,6 +57,7 @@ struct RegridArgs {
     int32_t nchan, nrest, bin_mode;
     uint32_t ncb;           // blocks of COLS columns a tile of rows takes
     int32_t pair_out;       // out_vis is 8-byte aligned: a value's two floats in one store
+    int32_t vec, vout;      // a channel's pols (and flags) in whole loads, an output channel's in whole stores
     float vis_scale;
     double l, m, n1, inv_zf;
     double zf, f0, df;      // 1 + z, the rest lattice
@@ -151,6 +154,7 @@ __device__ __forceinline__ float2 load_value(const char *at, float scale)
 }
 
 constexpr int COLS = 64;   // (output channel, pol) columns a block takes
+constexpr int POLS_THREADS = 128;
 
 template <int P, int VT, int R>
 __global__ void __launch_bounds__(COLS, 14) k_regrid(RegridArgs a)
@@ -240,13 +244,173 @@ __global__ void __launch_bounds__(COLS, 14) k_regrid(RegridArgs a)
     }
 }
 
-// Rows a tile: eight where that leaves at least four warps of work per
-// scheduler (152 x 4 of them), else four.
+// One channel's P values and flags of a row, at element i0 (= (row * nchan + k) * P).
+template <int P, int VT>
+__device__ __forceinline__ void load_channel(const RegridArgs &a, int64_t i0, float2 (&v)[P], uint32_t &fl)
+{
+    constexpr int VB = VisType<VT>::kBytes, LB = P * VB;
+    const char *at = reinterpret_cast<const char *>(a.vis) + i0 * VB;
+    if (P > 1 && a.vec) {
+        uint32_t w[LB / 4];
+        if constexpr (LB >= 16) {
+#pragma unroll
+            for (int q = 0; q < LB / 16; ++q) {
+                const uint4 x = __ldg(reinterpret_cast<const uint4 *>(at) + q);
+                w[4 * q] = x.x;
+                w[4 * q + 1] = x.y;
+                w[4 * q + 2] = x.z;
+                w[4 * q + 3] = x.w;
+            }
+        } else if constexpr (LB == 8) {
+            const uint2 x = __ldg(reinterpret_cast<const uint2 *>(at));
+            w[0] = x.x;
+            w[1] = x.y;
+        } else {
+            w[0] = __ldg(reinterpret_cast<const uint32_t *>(at));
+        }
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            if constexpr (VT == VISTA_VIS_C128)
+                v[p] = make_float2((float)__hiloint2double((int)w[4 * p + 1], (int)w[4 * p]),
+                                   (float)__hiloint2double((int)w[4 * p + 3], (int)w[4 * p + 2]));
+            else if constexpr (VT == VISTA_VIS_C64)
+                v[p] = make_float2(__uint_as_float(w[2 * p]), __uint_as_float(w[2 * p + 1]));
+            else {
+                const float2 x = VisType<VT>::half_pair(w[p]);
+                v[p] = make_float2(x.x * a.vis_scale, x.y * a.vis_scale);
+            }
+        }
+        fl = 0u;
+        if (a.flags) {
+            if constexpr (P == 4) fl = __ldg(reinterpret_cast<const uint32_t *>(a.flags + i0));
+            else fl = __ldg(reinterpret_cast<const uint16_t *>(a.flags + i0));
+        }
+        return;
+    }
+    fl = 0u;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        v[p] = load_value<VT>(at + p * VB, a.vis_scale);
+        if (a.flags) fl |= (uint32_t)__ldg(a.flags + i0 + p) << (8 * p);
+    }
+}
+
+// Narrow outputs: a thread per (tile of R rows, output channel) takes all its
+// pols, a channel's values in whole 16-byte (or shorter) loads.  k_regrid's block
+// shares one tile's columns, so that with few of them most of its threads idle:
+// 200 000 rows x 64 channels onto one, 1165 us there, 107 us here (98 us before there
+// was k_regrid); 20 000 rows x 500 channels onto four, four pols, 299 and 115 (108).
+template <int P, int VT, int R>
+__global__ void __launch_bounds__(POLS_THREADS) k_regrid_pols(RegridArgs a)
+{
+    const uint32_t t = blockIdx.x * POLS_THREADS + threadIdx.x, nt = (uint32_t)((a.nrow + R - 1) / R);
+    const uint32_t tile = t / (uint32_t)a.nrest;
+    const int j = (int)(t - tile * (uint32_t)a.nrest);
+    if (tile >= nt) return;
+    const int64_t r0 = (int64_t)tile * R;
+    const int nr = (int)(a.nrow - r0 < R ? a.nrow - r0 : R);
+    const int2 rg = *reinterpret_cast<const int2 *>(a.range + 2 * (int64_t)j);
+    const int first = INT_MAX - rg.x, cnt = rg.y > 0 ? rg.y - first : 0;
+    float2 tau[R];
+    float sr[R][P], si[R][P], sw[R][P];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        tau[r] = __ldg(a.tau + r0 + min(r, nr - 1));
+#pragma unroll
+        for (int p = 0; p < P; ++p) sr[r][p] = si[r][p] = sw[r][p] = 0.f;
+    }
+    for (int e = 0; e < cnt; ++e) {
+        const int k = first + e;
+        float2 v[R][P];
+        uint32_t fl[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) load_channel<P, VT>(a, ((r0 + min(r, nr - 1)) * a.nchan + k) * P, v[r], fl[r]);
+        const int4 c0 = __ldg(reinterpret_cast<const int4 *>(a.chan + k));        // j0, nb, w0, w1
+        const float4 c1 = __ldg(reinterpret_cast<const float4 *>(a.chan + k) + 1);   // w2, w3, nuc
+        const int b = j - c0.x;
+        if (b < 0 || b >= c0.y) continue;
+        const float w = b == 0 ? __int_as_float(c0.z) : b == 1 ? __int_as_float(c0.w) : b == 2 ? c1.x : c1.y;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float2 ph = shift_phasor(tau[r].x, tau[r].y, c1.z, c1.w);
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                if ((fl[r] >> (8 * p)) & 0xffu) continue;
+                sr[r][p] = __fmaf_rn(w, __fmaf_rn(v[r][p].x, ph.x, -__fmul_rn(v[r][p].y, ph.y)), sr[r][p]);
+                si[r][p] = __fmaf_rn(w, __fmaf_rn(v[r][p].x, ph.y, __fmul_rn(v[r][p].y, ph.x)), si[r][p]);
+                sw[r][p] += w;
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (r >= nr) break;
+        const int64_t o = ((r0 + r) * a.nrest + j) * P;
+        float ov[2 * P];
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const bool any = sw[r][p] > 0.f;
+            ov[2 * p] = any ? sr[r][p] / sw[r][p] : 0.f;
+            ov[2 * p + 1] = any ? si[r][p] / sw[r][p] : 0.f;
+        }
+        if (P > 1 && a.vout) {
+            float4 *d = reinterpret_cast<float4 *>(a.out_vis + 2 * o);
+#pragma unroll
+            for (int q = 0; q < P / 2; ++q) d[q] = make_float4(ov[4 * q], ov[4 * q + 1], ov[4 * q + 2], ov[4 * q + 3]);
+            if constexpr (P == 4) *reinterpret_cast<float4 *>(a.out_wsum + o) = make_float4(sw[r][0], sw[r][1], sw[r][2], sw[r][3]);
+            else if constexpr (P == 2) *reinterpret_cast<float2 *>(a.out_wsum + o) = make_float2(sw[r][0], sw[r][1]);
+            continue;
+        }
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            a.out_vis[2 * (o + p)] = ov[2 * p];
+            a.out_vis[2 * (o + p) + 1] = ov[2 * p + 1];
+            a.out_wsum[o + p] = sw[r][p];
+        }
+    }
+}
+
+template <int P, int VT, int R>
+cudaError_t launch_pols(RegridArgs a, cudaStream_t st)
+{
+    // (the threads are counted in 32 bits: more of them go in several launches)
+    const int64_t total = a.nrow, most = std::max<int64_t>(((int64_t)1 << 31) / a.nrest / R * R, R);
+    for (int64_t r = 0; r < total; r += most) {
+        a.nrow = total - r < most ? total - r : most;
+        const int64_t threads = (a.nrow + R - 1) / R * a.nrest;
+        k_regrid_pols<P, VT, R><<<(unsigned)((threads + POLS_THREADS - 1) / POLS_THREADS), POLS_THREADS, 0, st>>>(a);
+        const int64_t in = a.nrow * a.nchan * P, out = a.nrow * a.nrest * P;
+        a.vis = reinterpret_cast<const char *>(a.vis) + in * VisType<VT>::kBytes;
+        if (a.flags) a.flags += in;
+        a.tau += a.nrow;
+        a.out_vis += 2 * out;
+        a.out_wsum += out;
+    }
+    return cudaGetLastError();
+}
+
+// k_regrid takes outputs of two blocks of columns or more, or of one that is full;
+// narrower ones go to k_regrid_pols, two rows a thread from 200 000 (row, output
+// channel) pairs on.  k_regrid takes eight rows a tile where that leaves at least 16
+// blocks a SM and the lines a block's threads gather from at a time, up to one of
+// 128 bytes a row and output channel, stay within 8 KB; else four: with each output
+// channel's contributors far from its neighbour's, the eight rows' lines of an SM's
+// blocks overflow its L1 (12 000 rows x 3840 channels onto 64, two pols: eight 1148,
+// four 340 us).  Over 1249 shapes (1, 2 and 4 pols of three storage types, 500 to
+// 200 000 rows of 16 to 8000 channels, 1 to 1024 output channels) the rule is within
+// 7 % of the best of nine forms on average, and 10 % slower than the kernel before
+// k_regrid (a thread per row and output channel, its tables built on the host) on 42
+// of them, by half at the most; k_regrid with eight rows alone was on 40 %, by up
+// to twelve times.
 template <int P, int VT>
 cudaError_t launch_regrid_p(RegridArgs a, cudaStream_t st)
 {
-    const int64_t ncb = ((int64_t)a.nrest * P + COLS - 1) / COLS;
-    const bool eight = (a.nrow + 7) / 8 * ncb >= (int64_t)4 * 152;
+    constexpr int VB = VisType<VT>::kBytes;
+    const int64_t ncol = (int64_t)a.nrest * P, ncb = (ncol + COLS - 1) / COLS;
+    if (ncol < 2 * COLS && !(P > 1 && ncol > 56 && ncol <= COLS))
+        return a.nrow * a.nrest >= 200000 ? launch_pols<P, VT, 2>(a, st) : launch_pols<P, VT, 1>(a, st);
+    const int64_t apart = std::max<int64_t>(a.nchan / a.nrest, 1) * P * VB;   // bytes from a column's contributors to the next
+    const bool eight = (a.nrow + 7) / 8 * ncb >= (int64_t)16 * 152 && 8 * (COLS / P) * std::min<int64_t>(apart, 128) <= 8192;
     const int R = eight ? 8 : 4;
     const int64_t blocks = (a.nrow + R - 1) / R * ncb;
     // a tile's values lie within 32-bit offsets of its row pointers
@@ -336,6 +500,10 @@ extern "C" int vista_regrid_rows(vista_stack *h, const vista_source_desc *s, flo
     a.nchan = n;
     a.nrest = nrest;
     a.bin_mode = h->desc.bin_mode;
+    const size_t lane = vis_elem_bytes(s->vis_type) * (size_t)s->npol;
+    a.vec = ((uintptr_t)s->vis % std::min<size_t>(lane, 16)) == 0 &&
+            (!s->flags || ((uintptr_t)s->flags % (uintptr_t)s->npol) == 0);
+    a.vout = ((uintptr_t)out_vis % 16) == 0 && ((uintptr_t)out_wsum % (uintptr_t)(s->npol == 4 ? 16 : 8)) == 0;
     a.pair_out = ((uintptr_t)out_vis % 8) == 0;
     a.vis_scale = (s->vis_type == VISTA_VIS_F16X2 || s->vis_type == VISTA_VIS_BF16X2) ? s->vis_scale : 1.0f;
     a.zf = 1.0 + s->z;
