@@ -407,15 +407,15 @@ cudaError_t launch_regrid_p(RegridArgs a, cudaStream_t st)
 {
     constexpr int VB = VisType<VT>::kBytes;
     const int64_t ncol = (int64_t)a.nrest * P, ncb = (ncol + COLS - 1) / COLS;
-    if (ncol < 2 * COLS && !(P > 1 && ncol > 56 && ncol <= COLS))
+    // (k_regrid's offsets from its row pointers are 32-bit: longer rows go to the other form)
+    const bool far = (int64_t)a.nchan * P * VB > (int64_t)UINT32_MAX, full = P > 1 && ncol > 56 && ncol <= COLS;
+    if (far || (ncol < 2 * COLS && !full))
         return a.nrow * a.nrest >= 200000 ? launch_pols<P, VT, 2>(a, st) : launch_pols<P, VT, 1>(a, st);
     const int64_t apart = std::max<int64_t>(a.nchan / a.nrest, 1) * P * VB;   // bytes from a column's contributors to the next
     const bool eight = (a.nrow + 7) / 8 * ncb >= (int64_t)16 * 152 && 8 * (COLS / P) * std::min<int64_t>(apart, 128) <= 8192;
     const int R = eight ? 8 : 4;
     const int64_t blocks = (a.nrow + R - 1) / R * ncb;
-    // a tile's values lie within 32-bit offsets of its row pointers
-    if (blocks > (int64_t)INT_MAX || (int64_t)a.nchan * P * VisType<VT>::kBytes > (int64_t)UINT32_MAX)
-        return cudaErrorInvalidValue;
+    if (blocks > (int64_t)INT_MAX) return cudaErrorInvalidValue;   // (an output of more than 2^40 bytes)
     a.ncb = (uint32_t)ncb;
     if (eight)
         k_regrid<P, VT, 8><<<(unsigned)blocks, COLS, 0, st>>>(a);
