@@ -92,6 +92,25 @@ __device__ __forceinline__ double2 phasor64(double t)   // exp(2 pi i t)
     return make_double2(c, s);
 }
 
+// The phasors of one row (delay tau) at a chunk's nch <= 32 channels, handed to
+// take(k, phasor): by recurrence from the chunk's first channel where the axis is
+// linear, else one by one.
+template <typename F>
+__device__ __forceinline__ void chunk_phasors(const SrcDev &S, const ChanD *cd, int nch, double tau, F &&take)
+{
+    if (S.linear) {
+        double2 ph = phasor64(tau * (cd[0].nu * (1.0 / C_LIGHT)));
+        const double2 st = phasor64(tau * S.step_c);
+        for (int k = 0;; ++k) {
+            take(k, ph);
+            if (k == nch - 1) break;
+            ph = make_double2(ph.x * st.x - ph.y * st.y, ph.x * st.y + ph.y * st.x);
+        }
+    } else {
+        for (int k = 0; k < nch; ++k) take(k, phasor64(tau * (cd[k].nu * (1.0 / C_LIGHT))));
+    }
+}
+
 template <int P>
 struct __align__(16) Warp64 {
     double2 ph[32][33];   // [row][channel], padded: both phases' accesses are conflict-free
@@ -186,20 +205,9 @@ __global__ void __launch_bounds__(32 * WARPS64, 3) stack_fp64_runs(RunArgs a)
                 for (int p = 0; p < P; ++p) T.W[lane][p] = widen_exact(rec.W[P == 4 ? p : 2 * p]);
                 const double *x = S.uvw + 3 * (int64_t)rec.row;   // the stored baseline: the delay of Eq. 2
                 const double tau = x[0] * S.l + x[1] * S.m + x[2] * S.n1;
-                if (S.linear) {
-                    double2 ph = phasor64(tau * (cd[0].nu * (1.0 / C_LIGHT)));
-                    const double2 st = phasor64(tau * S.step_c);
-                    for (int k = 0;; ++k) {
-                        T.ph[lane][k] = make_double2(ph.x, rec.fold ? -ph.y : ph.y);
-                        if (k == nch - 1) break;
-                        ph = make_double2(ph.x * st.x - ph.y * st.y, ph.x * st.y + ph.y * st.x);
-                    }
-                } else {
-                    for (int k = 0; k < nch; ++k) {
-                        const double2 ph = phasor64(tau * (cd[k].nu * (1.0 / C_LIGHT)));
-                        T.ph[lane][k] = make_double2(ph.x, rec.fold ? -ph.y : ph.y);
-                    }
-                }
+                chunk_phasors(S, cd, nch, tau, [&](int k, double2 ph) {
+                    T.ph[lane][k] = make_double2(ph.x, rec.fold ? -ph.y : ph.y);
+                });
             }
             __syncwarp();
             // the rows' values and flags are loaded one row ahead
@@ -280,7 +288,45 @@ cudaError_t launch_vt(const RunArgs &a, int npol, cudaStream_t st)
     }
 }
 
+// The phasors and cells of one window, as the stacking kernel forms them, at the
+// channels that reach the cube: one thread per row.
+__global__ void __launch_bounds__(128) debug_fp64(RunArgs a, int src, double *ph_out, int32_t *cell_out)
+{
+    const SrcDev &S = a.srcs[src];
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // processing order
+    if (i >= S.nrow) return;
+    const RowRec rec = a.recs[S.rec_off + i];
+    const double *x = S.uvw + 3 * (int64_t)rec.row;   // the stored baseline: the delay of Eq. 2
+    const double tau = x[0] * S.l + x[1] * S.m + x[2] * S.n1;
+    for (int c = 0; c < S.nchunk; ++c) {
+        const int k0 = S.k_lo + 32 * c;
+        const ChanD *cd = a.chd + S.chan_off + 32 * c;
+        const int2 cc = a.ccells[S.cell_off + (int64_t)c * S.nrow + i];
+        chunk_phasors(S, cd, min(32, S.k_hi - k0), tau, [&](int k, double2 ph) {
+            if (cd[k].nb <= 0) return;
+            const int64_t o = (int64_t)rec.row * S.nchan + k0 + k;
+            if (ph_out) {
+                ph_out[2 * o] = ph.x;
+                ph_out[2 * o + 1] = ph.y;
+            }
+            if (cell_out) {
+                const int cid = cc.y == CC_NOCHANGE ? cc.x
+                                : cc.y != CC_MIXED  ? chunk_cell_step(cc, k, a.g.nu)
+                                                    : cell_exact(S.guvw, rec.row, rec.fold != 0u, cd + k, a.g.nu, a.g.nv);
+                cell_out[2 * o] = cid < 0 ? -1 : cid % a.g.nu;
+                cell_out[2 * o + 1] = cid < 0 ? -1 : cid / a.g.nu;
+            }
+        });
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_debug_fp64(const RunArgs &a, int src, int64_t nrow, double *ph, int32_t *cells, cudaStream_t st)
+{
+    if (nrow > 0) debug_fp64<<<(unsigned)((nrow + 127) / 128), 128, 0, st>>>(a, src, ph, cells);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_fp64(const RunArgs &a, int key, cudaStream_t st)
 {

@@ -268,6 +268,8 @@ cudaError_t launch_prepare(const RunArgs &a, cudaStream_t st, int *nlaunch = nul
 cudaError_t launch_mixed(const RunArgs &a, int key, int warps_per_cta, int prefetch, cudaStream_t st);
 // The FP64 stacking kernel of one class (chunks of 32 channels), same key.
 cudaError_t launch_fp64(const RunArgs &a, int key, cudaStream_t st);
+// The FP64 form's phasors and cells of window src (nrow rows), exported.
+cudaError_t launch_debug_fp64(const RunArgs &a, int src, int64_t nrow, double *ph, int32_t *cells, cudaStream_t st);
 // Mixed cube: move every FP32 partial into the FP64 master and clear it.
 inline size_t moved_bytes(int64_t n) { return (size_t)((n + 31) / 32) * sizeof(uint32_t); }
 cudaError_t launch_fold(void *cube, double *master, uint32_t *moved, int64_t n, cudaStream_t st);

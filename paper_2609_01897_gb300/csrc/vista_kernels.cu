@@ -1,7 +1,7 @@
 // libvista kernels over the cube, for sm_103a.
 //
 //   (the stacking kernels are in vista_stack.cuh and vista_fp64.cu)
-//   debug_*       the phasors and cells of the two forms, exported
+//   debug_mixed   the mixed form's phasors and cells, exported
 //   unpack        cube -> caller arrays
 //   zero          the touched entries back to zero
 //   sparse_*      the touched entries -> caller arrays
@@ -55,43 +55,6 @@ __global__ void debug_mixed(RunArgs a, int src, double *ph_out, int32_t *cell_ou
                 cell_out[2 * o] = ok ? iu : -1;
                 cell_out[2 * o + 1] = ok ? iv : -1;
             }
-        }
-    }
-}
-
-// Debug export of the FP64 form's phasors and cells: the FP64 phase of every
-// channel that reaches the cube (the stacking kernel's recurrence is seeded
-// from the same expression at each chunk of 32 channels) and the FP64 cell
-// rule, one thread per row.
-__global__ void __launch_bounds__(128) debug_fp64(RunArgs a, int src, double *ph_out, int32_t *cell_out)
-{
-    const SrcDev &S = a.srcs[src];
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= S.nrow) return;
-    const double *uvw = S.uvw + 3 * r;     // the stored baseline: the delay of Eq. 2
-    const double tau = uvw[0] * S.l + uvw[1] * S.m + uvw[2] * S.n1;
-    double u = S.guvw[3 * r], v = S.guvw[3 * r + 1];   // the gridding baseline (Eq. 1)
-    if (a.g.fold && (v < 0.0 || (v == 0.0 && u < 0.0))) {
-        u = -u;
-        v = -v;
-    }
-    const ChanD *cd = a.chd + S.chan_off;
-    for (int k = S.k_lo; k < S.k_hi; ++k) {
-        const ChanD &c = cd[k - S.k_lo];
-        if (c.nb <= 0) continue;
-        const int64_t o = r * S.nchan + k;
-        if (ph_out) {
-            const double t = tau * (c.nu * (1.0 / C_LIGHT));
-            double s, co;
-            sincospi(2.0 * (t - floor(t)), &s, &co);
-            ph_out[2 * o] = co;
-            ph_out[2 * o + 1] = s;
-        }
-        if (cell_out) {
-            const int iu = axis_cell64(u, c.su, a.g.nu), iv = axis_cell64(v, c.sv, a.g.nv);
-            const bool on = iu >= 0 && iv >= 0;
-            cell_out[2 * o] = on ? iu : -1;
-            cell_out[2 * o + 1] = on ? iv : -1;
         }
     }
 }
@@ -487,10 +450,7 @@ cudaError_t launch_debug(const RunArgs &a, int ns, int src, int fp64, double *ph
     if (e != cudaSuccess) return e;
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
-    if (fp64) {
-        if (S.nrow > 0) debug_fp64<<<(unsigned)((S.nrow + 127) / 128), 128, 0, st>>>(a, src, ph, cells);
-        return cudaGetLastError();
-    }
+    if (fp64) return launch_debug_fp64(a, src, S.nrow, ph, cells, st);
     const int64_t tasks = S.nrow * S.nchunk;
     if (tasks == 0) return cudaSuccess;
     const int64_t blocks = (tasks + 3) / 4;
