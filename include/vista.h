@@ -158,12 +158,12 @@ typedef struct {
  *                   records are staged in shared memory).
  *   chans_per_lane  channels per lane in one item (item = 32 x this many
  *                   channels; 1, 2 or 4).
- *   warps_per_cta   warps per block of the stacking kernel.
+ *   warps_per_cta   warps per block of the stacking kernel (1, 2, 4 or 8;
+ *                   the kernel's blocks hold at most four, so 8 runs as 4).
  *   sort_rows       1: order rows by uv cell before stacking (fewer
  *                   global reductions), 0: stack in input order.
- *   prefetch_rows   visibility rows each warp keeps in flight (2, 4 or 8
- *                   with one channel per lane, 2 or 4 with two, 2 with
- *                   four). */
+ *   prefetch_rows   visibility rows each warp keeps in flight (2, 4 or 8),
+ *                   besides the two it works on. */
 typedef struct {
     int32_t rows_per_item, chans_per_lane, warps_per_cta, sort_rows, prefetch_rows;
 } vista_tuning;
@@ -343,7 +343,7 @@ int vista_get_timing(vista_stack *h, vista_timing *out);
 
 /* Autotuner of the launch shape (mixed precision).  Times the queued source
  * set under up to `budget` candidate shapes (0 = all of a fixed list: rows
- * per item 32-96, one or two channels per lane, 2-8 warps per block, 2-8
+ * per item 32-96, one or two channels per lane, 2-4 warps per block, 2-8
  * rows in flight; the current shape first), `reps` runs each (0 = 2), by
  * the event-timed device work of vista_run(), and keeps the fastest as the
  * handle's tuning (also returned in *best, which may be NULL).  The trial

@@ -32,8 +32,7 @@ std::vector<LaunchCfg> candidates(const LaunchCfg &cur)
     for (int cpl : {1, 2})
         for (int pf : pfs)
             for (int r : rows) add(r, cpl, 4, pf);
-    for (int r : rows) add(r, 1, 2, 4);
-    for (int r : rows) add(r, 1, 8, 4);
+    for (int r : rows) add(r, 1, 2, 4);   // (blocks hold at most four warps)
     return c;
 }
 
