@@ -36,20 +36,18 @@ __device__ __forceinline__ bool is_moved(uint32_t word, int64_t i) { return (wor
 // is the double to about 2^-47 relative, less where lo falls below the
 // normal floats).  Integer and FP32 operations only.  Magnitudes below 2^-126
 // give (0, 0): zero, and values far below any sum of weights or visibilities.
-// Magnitudes from 2^128 on, and infinities, give (infinity, 0), NaN (NaN, 0).
+// Magnitudes from 2^128 on, infinities and NaNs give a pair that is not finite
+// (the exponent saturates; with a branch for them the subtraction of an FP64 cube
+// of 1.7e7 entries took 290 us instead of 263).
 __device__ __forceinline__ float2 split_double(double d)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(d);
     const int e = (int)((b >> 52) & 0x7ff);
     if (e < 897) return make_float2(0.f, 0.f);
-    const unsigned sign = (unsigned)(b >> 63) << 31;
-    if (__builtin_expect(e > 1150, 0)) {
-        const bool nan = e == 0x7ff && (b & 0xfffffffffffffull) != 0;
-        return make_float2(__uint_as_float(sign | (nan ? 0x7fc00000u : 0x7f800000u)), 0.f);
-    }
-    const unsigned hi_bits = sign | ((unsigned)(e - 896) << 23) | (unsigned)((b >> 29) & 0x7fffffu);
+    const unsigned sign = (unsigned)(b >> 63) << 31, ef = (unsigned)min(e - 896, 255) << 23;
+    const unsigned hi_bits = sign | ef | ((unsigned)(b >> 29) & 0x7fffffu);
     // the low 29 mantissa bits times 2^-52 (exact), times 2^(e - 1023)
-    const float lo = (__uint2float_rn((unsigned)(b & 0x1fffffffu)) * 0x1p-52f) * __int_as_float((e - 896) << 23);
+    const float lo = (__uint2float_rn((unsigned)(b & 0x1fffffffu)) * 0x1p-52f) * __uint_as_float(ef);
     return make_float2(__uint_as_float(hi_bits), sign ? -lo : lo);
 }
 

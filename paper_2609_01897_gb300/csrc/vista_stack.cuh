@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(KMAX_THREADS, (min_blocks<P>())) stack_mixed(R
             // sum L / (32 / 4 P) and the entry's sums go out as one reduction of
             // adjacent floats; the counts of a pol pair are added as 16-bit halves.
             // Staged and drained, such runs would meet in the same entries all the
-            // same, at three times the instructions (four pols: 17.3 -> 14.4 ms on
+            // same, at three times the instructions (four pols: 17.3 -> 14.4 ms then on
             // the four-pol windows of an archive stack; two pols: no gain).
             auto reduce_runs = [&](int c, bool fl) {
                 constexpr int N = 4 * P, LPS = 32 / N;   // sums, lanes per sum in the end
@@ -497,8 +497,11 @@ __global__ void __launch_bounds__(KMAX_THREADS, (min_blocks<P>())) stack_mixed(R
                 const bool fl = cid != cell;
                 const unsigned bal = __ballot_sync(0xffffffffu, fl);
                 if (P == 4 && narrow && __popc(bal) >= 8) {
-                    // most lanes end a run, as a rule in one cell: the warp adds the
-                    // runs up and writes the one or two entries itself
+                    // many lanes end a run, as a rule in one cell: the warp adds the
+                    // runs up and writes the one or two entries itself (from how many
+                    // on hardly matters, the lanes end their runs together or nearly
+                    // alone: 1, 4, 8, 16 and 32 give 12.52 to 12.56 ms on the four-pol
+                    // windows of an archive stack; never, 13.27 ms)
                     const int c0 = __shfl_sync(0xffffffffu, cell, __ffs(bal) - 1);
                     if (c0 >= 0 && __all_sync(0xffffffffu, !fl || cell == c0)) {
                         reduce_runs(c0, fl);
