@@ -243,7 +243,10 @@ int vista_regrid_rows(vista_stack *h, const vista_source_desc *src, float *out_v
  * stream through two device staging slots in waves of about a quarter of
  * their bytes (64 MB to 2 GB): the copies of one wave, on four copy streams,
  * run while the wave before is stacked (the paper's read -> compute overlap,
- * Sec. 3.1 and 3.3).  E_STATE if nothing is queued,
+ * Sec. 3.1 and 3.3).  In either precision the rows are put in uv-cell order
+ * first, in device buffers of the handle that grow as runs need them (about 52
+ * bytes a row and 9 a row and 32-channel chunk; E_NOMEM if they cannot be
+ * had).  E_STATE if nothing is queued,
  * E_RANGE if a channel would touch more than VISTA_MAX_BINS rest bins. */
 int vista_run(vista_stack *h);
 

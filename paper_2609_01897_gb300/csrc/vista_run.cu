@@ -475,7 +475,7 @@ extern "C" int vista_run(vista_stack *h)
         const SrcHost &s = h->pending[(size_t)i];
         const Plan &pl = plans[(size_t)i];
         if (s.d.nrow == 0 || pl.k_hi <= pl.k_lo) continue;
-        // four pols x four channels per lane does not fit the register budget
+        // (windows of four pols take chunks of at most 64 channels)
         const int cap = s.d.npol == 4 ? std::min(2, (int)cfg.chans_per_lane) : (int)cfg.chans_per_lane;
         const int ns = fp64 ? 1 : choose_ns(pl.k_hi - pl.k_lo, cap);
         ns_of[(size_t)i] = ns;
