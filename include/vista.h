@@ -82,7 +82,7 @@ typedef struct vista_stack vista_stack;   /* opaque handle */
  *              body, an FP32 cube whose entries are moved into an FP64 master
  *              cube at checkpoints spread over the drains and folded into it
  *              wholly after a run once 64 visibilities per cube entry have
- *              been stacked since the last fold (measured within 6e-7
+ *              been stacked since the last fold (measured within 7e-7
  *              relative on every entry of a 1.9e11-visibility stack stacked
  *              twice); VISTA_PREC_FP64: FP64 throughout with an FP64 cube.
  *   hermitian_fold  1: rows with v < 0 (or v == 0, u < 0) are negated and

@@ -21,7 +21,7 @@
 // L2 twice); the warp then synchronises before a group's values are read and
 // before their ring slots are refilled.
 //
-// The kernel is bound by the issue and latency of its instructions (57 to 62 %
+// The kernel is bound by the issue and latency of its instructions (57 to 64 %
 // issue with 15 warps an SM) before it is bound by HBM, so it is built to spend
 // few instructions per (row, 32 channels):
 //  - the arithmetic is in packed FP32 pairs (one instruction per pair): with
@@ -52,10 +52,10 @@
 //
 // Measured, before (values through predicated scalar arithmetic, one row at a
 // time, runs written unmerged) and now, kernel time: a compact array's stack,
-// two pols of complex64, 5.2e8 visibilities, 1.96 -> 1.61 ms; an archive
-// stack, 1.2e10 visibilities of two and four pols, 28.5 -> 23.2 ms (4.8 TB/s);
-// wideband FP16, 7.5e8 visibilities, 2.75 -> 1.90 ms; long baselines in BF16,
-// 4.6e8 visibilities, 1.46 -> 1.14 ms.  Per (row, 32 channels) of two pols a
+// two pols of complex64, 5.2e8 visibilities, 1.96 -> 1.56 ms; an archive
+// stack, 1.2e10 visibilities of two and four pols, 28.5 -> 22.2 ms (5.1 TB/s);
+// wideband FP16, 7.5e8 visibilities, 2.75 -> 1.89 ms; long baselines in BF16,
+// 4.6e8 visibilities, 1.46 -> 1.13 ms.  Per (row, 32 channels) of two pols a
 // warp issues about 78 instructions where no run ends (99 before the row loop
 // lost its branches), 112 on the compact array's stack (178 before).
 #pragma once
