@@ -312,6 +312,7 @@ __global__ void __launch_bounds__(SPARSE_THREADS) sparse_write_kernel(const void
     __shared__ int ws[SPARSE_WARPS];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t base = (int64_t)blockIdx.x * SPARSE_TILE;
+    const bool sums = sum_wv || sum_w || sum_wvv;
     int64_t pos = tile_off[blockIdx.x];
     for (int k = 0; k < SPARSE_ROUNDS; ++k) {
         const int64_t i = base + (int64_t)k * SPARSE_THREADS + threadIdx.x;
@@ -327,8 +328,9 @@ __global__ void __launch_bounds__(SPARSE_THREADS) sparse_write_kernel(const void
         if (c != 0u) {
             const int64_t q = pos + before + __popc(bal & ((1u << lane) - 1u));
             if (q < cap) {
-                float e[4];
-                if (fp64) {
+                float e[4] = {0.f, 0.f, 0.f, 0.f};
+                if (!sums) {   // (the index and the count alone)
+                } else if (fp64) {
                     RawEntry<true> r;
                     r.load(cube, nullptr, false, i);
                     r.value(e);

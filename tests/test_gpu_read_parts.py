@@ -57,6 +57,26 @@ def test_parts_equal_the_whole(V, fp64, f64, nu, nrest, npol, nrow, runs):
         st.close()
 
 
+@pytest.mark.parametrize("fp64", [False, True])
+def test_sparse_parts_equal_the_whole(V, fp64):
+    import ctypes as C
+    st = _stacked(V, V.PREC_FP64 if fp64 else V.PREC_MIXED, 20, 23, 2, 2000, 3)
+    try:
+        whole = st.read_cube_sparse(device=True)
+        n, got = C.c_int64(0), int(whole["index"].shape[0])
+        assert got > 1000
+        for which in ((), ("count",), ("sum_w",), ("sum_wvv", "count"), ("sum_wv",)):
+            part = {k: torch.full_like(x, 7) for k, x in whole.items()}
+            ptr = {k: (x.data_ptr() if k == "index" or k in which else None) for k, x in part.items()}
+            rc = V.lib().vista_read_cube_sparse(st.h, got, ptr["index"], ptr["sum_wv"], ptr["sum_w"], ptr["sum_wvv"],
+                                                ptr["count"], C.byref(n), 1)
+            assert rc == 0 and n.value == got
+            for k, x in part.items():
+                assert torch.equal(x, whole[k] if ptr[k] else torch.full_like(x, 7)), (which, k)
+    finally:
+        st.close()
+
+
 def test_counts_alone_do_not_read_the_sums(V):
     st = _stacked(V, V.PREC_FP64, 256, 64, 4, 40000, 1)
     try:
